@@ -432,7 +432,7 @@ def run_gpu(args):
     else:
         fp32_peak = 152 * 128 * 2 * pk.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
         peak_note = f"FP32 derived (152 SMs x 128 lanes x 2 flop x max clock), not measured: {pk_err}"
-    roof = {"kernel": "k_m2l_f32w", "bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
+    roof = {"kernel": "k_m2l_mma", "bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
             "frac": achieved / fp32_peak, "traffic": None, "peak_note": peak_note,
             "work": f"{n_eval:.3e} kernel entries x {flops_per_eval:.0f} flop per matvec", "m2l_ms": m2l_ms}
     if pk_alu:

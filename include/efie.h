@@ -85,7 +85,7 @@ typedef struct {
                         in every product, which is faster than streaming them); 1 always
                         evaluate; 2 always keep (EFIE_ENOMEM if they do not fit) */
   int m2l_batch;     /* M2L of a product with several right-hand sides in the mixed form:
-                        0 automatic (tensor cores when q <= 10, else FP32 on the CUDA cores),
+                        0 automatic (split TF32 on the tensor cores),
                         1 FP32 on the CUDA cores, 2 tensor cores (split TF32 with FP32
                         accumulation, q <= 10; EFIE_EINVAL at setup otherwise) */
   int leaf_dense;    /* 0: the paper's block tree (Algorithm 1); 1: leaf-level variant, in which

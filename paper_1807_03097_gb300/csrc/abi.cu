@@ -44,7 +44,8 @@ void release_device(Ctx *c) {
   dfree(c, c->d_V); dfree(c, c->d_H); dfree(c, c->d_h); dfree(c, c->d_h2); dfree(c, c->d_part); dfree(c, c->d_gs);
   dfree(c, c->d_w); dfree(c, c->d_r); dfree(c, c->d_b); dfree(c, c->d_sol);
   dfree(c, c->d_xB); dfree(c, c->d_yB); dfree(c, c->d_xsB); dfree(c, c->d_ysB); dfree(c, c->d_ysnB);
-  dfree(c, c->d_momB); dfree(c, c->d_srcB); dfree(c, c->d_accB); dfree(c, c->d_locB); dfree(c, c->d_tc_err);
+  dfree(c, c->d_momB); dfree(c, c->d_srcB); dfree(c, c->d_accB); dfree(c, c->d_locB); dfree(c, c->d_moreB);
+  dfree(c, c->d_tc_err);
   c->batch_cap = 0;
   c->kr = 0;
   c->part_cap = 0;

@@ -17,6 +17,7 @@ constexpr int kMaxGeoDeg = 8;     // NURBS degree limit of the device evaluator
 constexpr int kMaxGeoCp = 64;     // control points per direction
 constexpr int kMaxQ1 = 17;        // q + 1 interpolation points per direction
 constexpr int kMaxP1 = 7;         // p + 1 Bernstein functions per direction
+constexpr int kMmaMaxRhs = 7;     // most right-hand sides of a batch in k_m2l_mma beside k_m2l_tc
 
 // One NURBS patch as the device sees it: offsets into the packed knot and homogeneous
 // control point arrays.
@@ -125,6 +126,7 @@ struct Ctx {
   int h_resB_cap = 0;
   double2 *d_xB = nullptr, *d_yB = nullptr, *d_xsB = nullptr, *d_ysB = nullptr, *d_ysnB = nullptr;
   float2 *d_momB = nullptr, *d_srcB = nullptr, *d_accB = nullptr, *d_locB = nullptr;
+  float2 *d_moreB = nullptr;  // [m2l_split - 1][ncl][nI][4 kMmaMaxRhs]: further splits of d_accB
   int *d_tc_err = nullptr;   // set by a tensor-core M2L whose pipeline wait ran out
   int *d_near_ptr = nullptr, *d_near_src = nullptr;  // CSR by target element
   double2 *d_nblk = nullptr;  // [nnear][nb (col)][nb (row)]
@@ -146,7 +148,8 @@ struct Ctx {
   // work vectors (FP32 path)
   float2 *d_momf = nullptr, *d_locf = nullptr;
   float4 *d_srcf = nullptr;   // [ncl][nI][2]: (u_x, u_y), (u_z, nu) folded source fields
-  float4 *d_accf = nullptr;   // [ncl][nI][2]: M2L results, same layout
+  float4 *d_accf = nullptr;   // [m2l_split][ncl][nI][2]: M2L results, same layout
+  int m2l_split = 1;          // splits of the source lists in k_m2l_mma
   float4 *d_nodeX4 = nullptr; // [ncl][nI] node offsets from the cluster centre (x, y, z, 0)
   float4 *d_pgeo = nullptr;   // per far pair (CSR order): centre offset d = c_t - c_s, r0 = |d|
   float2 *d_pph = nullptr;    // per far pair: e^{i kappa r0} / (4 pi)
@@ -221,6 +224,19 @@ efie_status dev_near_apply_batch(Ctx *c, int R, const double2 *xs, double2 *ysn,
 efie_status dev_matvec_batch(Ctx *c, int R, const double2 *const *X, double2 *const *Y, bool superspace = false);
 // R independent GMRES solves advanced in lockstep, one batched matvec per step
 size_t gmres_batch_bytes_per_system(const Ctx *c);
+// M2L of one or a few right-hand sides with the kernel entries in mma.sync operands (m2l_mma.cu):
+// fields src[(cluster nI + node) ld + 4 r + f], results acc likewise (split 0 of the source lists)
+// and more[(split - 1) slab + (cluster nI + node) ldm + 4 r + f]
+struct MmaArgs {
+  int R, ld, split;
+  const float2 *src;
+  float2 *acc, *more;
+  int ldm;
+  size_t slab;
+};
+int m2l_mma_splits(const Ctx *c);
+int m2l_mma_rhs(const Ctx *c);  // right-hand sides up to which a batch takes it
+efie_status launch_m2l_mma(Ctx *c, cudaStream_t st, const MmaArgs &A);
 // tensor-core M2L of a batch (m2l_tc.cu)
 bool m2l_tc_supported(const Ctx *c);
 efie_status m2l_tc_prepare(Ctx *c);

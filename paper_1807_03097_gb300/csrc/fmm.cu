@@ -327,11 +327,10 @@ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
   return *reinterpret_cast<float2 *>(&D);
 }
 
-// FP32 M2L, one warp per target cluster; lane owns target nodes m = lane + j T (j < NT,
-// T = ceil(nI / NT) <= 32) and sweeps the source nodes of every admissible source cluster two
-// at a time, so that the kernel values of two entries (m, m'), (m, m'+1) are generated and
-// applied with packed FP32 instructions (fma / add / mul .f32x2 on the pair).  With x_t, x_s
-// the node offsets from the cluster centres, d = c_t - c_s and r0 = |d|:
+// FP32 M2L over unordered admissible pairs: every coupling tile K_ts is evaluated once and
+// applied in both directions, acc_t += K_ts w_s and acc_s += K_ts^T w_t (K is symmetric in the
+// two clusters: it depends on |x_t - x_s| only).  With x_t, x_s the node offsets from the cluster
+// centres, d = c_t - c_s and r0 = |d|, G = e^{i kappa r0}/(4 pi) * e^{i phase} / r and
 //   MODE 0 (direct): r^2 = |u|^2 + |x_s|^2 - 2 u.x_s with u = d + x_t, phase = kappa r -
 //     kappa r0; used when the host has checked that kappa * max r * 2^-24 < 5e-6 (a fixed
 //     perturbation of the matrix of at most about 2e-5 rad per entry);
@@ -340,189 +339,6 @@ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
 //     phase = kappa (r - r0) = num / ((r + r0) / kappa); the host has checked that every phase
 //     lies within +-100 pi;  MODE 2: MODE 1 plus a two-constant Cody-Waite reduction of the
 //     phase to [-pi, pi] before the hardware sine / cosine.
-// G = e^{i kappa r0}/(4 pi) * e^{i phase} / r.  The pair factor e^{i kappa r0}/(4 pi) is
-// applied to the source fields while they are staged in shared memory.  Staging of a source
-// pair k (nodes 2k, 2k+1; an odd last node is paired with a copy of itself with zero fields):
-//   sC[2k]   = (-2x_e, -2x_o, -2y_e, -2y_o),  sC[2k+1] = (-2z_e, -2z_o, b_e, b_o)
-//     (b = |x_s|^2 in MODE 0, |x_s|^2 - 2 d.x_s otherwise),
-//   sF[6k..6k+5] = Re w (fields 0-1, 2-3), Im w (0-1, 2-3), -Im w (0-1, 2-3), each float4 holding
-//     (field f even node, field f odd node, field f+1 even node, field f+1 odd node).
-// Per pair the packed partial sums (even and odd source nodes separately) are folded and
-// added to running sums over all source clusters with two-sum (compensated) addition; the
-// running sums and their compensation terms live in shared memory ([NT][16][32 lanes] per warp,
-// touched once per source cluster), which keeps the registers for the inner loop.
-template <int NT, int MODE>
-__global__ void __launch_bounds__(128, (NT <= 3 ? 4 : 2)) k_m2l_f32w(const int *__restrict__ targets, int ntarget,
-                                                  const int *__restrict__ fptr, const int *__restrict__ fsrc,
-                                                  const float4 *__restrict__ pgeo, const float2 *__restrict__ pph,
-                                                  int nI, float kappa, const float4 *__restrict__ nodeX4,
-                                                  const float4 *__restrict__ src, float4 *__restrict__ acc) {
-  extern __shared__ float4 sm4[];
-  const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int wg = blockIdx.x * (blockDim.x >> 5) + wib;
-  if (wg >= ntarget) return;
-  const int NSP = (nI + 1) >> 1;  // source node pairs
-  float4 *sT = sm4 + (size_t)wib * (nI + 8 * NSP + 4 * 32 * NT);
-  float4 *sC = sT + nI;   // [2 NSP]
-  float4 *sF = sC + 2 * NSP;  // [6 NSP]
-  float *sA = reinterpret_cast<float *>(sF + 6 * NSP);  // [NT][16][32]: running sums, compensation
-  const int t = targets[wg];
-  const int T = (nI + NT - 1) / NT;
-  for (int i = lane; i < nI; i += 32) sT[i] = nodeX4[(size_t)t * nI + i];
-#pragma unroll
-  for (int j = 0; j < NT; ++j)
-#pragma unroll
-    for (int q = 0; q < 16; ++q) sA[(j * 16 + q) * 32 + lane] = 0.f;
-  const float inv2pi = 0.15915494309189535f, c1 = 6.28318548202514648f, c2 = -1.7484555e-7f;
-  const float kinv = 1.f / kappa;
-  for (int k = fptr[t]; k < fptr[t + 1]; ++k) {
-    const int s = fsrc[k];
-    const float4 g = pgeo[k];
-    const float2 ph = pph[k];
-    __syncwarp();
-    for (int i = lane; i < 2 * NSP; i += 32) {
-      const int kp = i >> 1, e = i & 1;
-      const int n = min(2 * kp + e, nI - 1);
-      const bool real = 2 * kp + e < nI;
-      const float4 x = nodeX4[(size_t)s * nI + n];
-      float4 u = make_float4(0.f, 0.f, 0.f, 0.f), v = u;
-      if (real) {
-        u = src[2 * ((size_t)s * nI + n)];
-        v = src[2 * ((size_t)s * nI + n) + 1];
-      }
-      const float bb = MODE == 0 ? x.x * x.x + x.y * x.y + x.z * x.z
-                                 : x.x * x.x + x.y * x.y + x.z * x.z - 2.f * (g.x * x.x + g.y * x.y + g.z * x.z);
-      // fields w_f = ph * (u.xy, u.zw, v.xy, v.zw)
-      const float wr[4] = {ph.x * u.x - ph.y * u.y, ph.x * u.z - ph.y * u.w, ph.x * v.x - ph.y * v.y,
-                           ph.x * v.z - ph.y * v.w};
-      const float wi[4] = {ph.x * u.y + ph.y * u.x, ph.x * u.w + ph.y * u.z, ph.x * v.y + ph.y * v.x,
-                           ph.x * v.w + ph.y * v.z};
-      float *c = reinterpret_cast<float *>(sC + 2 * kp);
-      c[e] = -2.f * x.x;
-      c[2 + e] = -2.f * x.y;
-      c[4 + e] = -2.f * x.z;
-      c[6 + e] = bb;
-      float *f = reinterpret_cast<float *>(sF + 6 * kp);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int o = (q >> 1) * 4 + (q & 1) * 2 + e;
-        f[o] = wr[q];
-        f[8 + o] = wi[q];
-        f[16 + o] = -wi[q];
-      }
-    }
-    __syncwarp();
-    // per-lane constants of this pair for each target node
-    float2 U[NT][4];
-#pragma unroll
-    for (int j = 0; j < NT; ++j) {
-      const int mi = lane + j * T;
-      const float4 x = sT[(lane < T && mi < nI) ? mi : 0];
-      float ax, ay, az, aa;
-      if (MODE == 0) {
-        ax = g.x + x.x;
-        ay = g.y + x.y;
-        az = g.z + x.z;
-        aa = ax * ax + ay * ay + az * az;
-      } else {
-        ax = x.x;
-        ay = x.y;
-        az = x.z;
-        aa = x.x * x.x + x.y * x.y + x.z * x.z + 2.f * (g.x * x.x + g.y * x.y + g.z * x.z);
-      }
-      U[j][0] = make_float2(ax, ax);
-      U[j][1] = make_float2(ay, ay);
-      U[j][2] = make_float2(az, az);
-      U[j][3] = make_float2(aa, aa);
-    }
-    const float2 r0sq = make_float2(g.w * g.w, g.w * g.w), nkr0 = make_float2(-kappa * g.w, -kappa * g.w);
-    const float2 kap2 = make_float2(kappa, kappa), kinv2 = make_float2(kinv, kinv);
-    const float2 r0k = make_float2(g.w * kinv, g.w * kinv);
-    float2 are[NT][4], aim[NT][4];  // this pair's packed partial sums (even, odd source nodes)
-#pragma unroll
-    for (int j = 0; j < NT; ++j)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) are[j][q] = aim[j][q] = make_float2(0.f, 0.f);
-#pragma unroll 1
-    for (int kp = 0; kp < NSP; ++kp) {
-      const float4 ca = sC[2 * kp], cb = sC[2 * kp + 1];
-      const float2 sx = make_float2(ca.x, ca.y), sy = make_float2(ca.z, ca.w), sz = make_float2(cb.x, cb.y),
-                   sb = make_float2(cb.z, cb.w);
-      float2 gr[NT], gi[NT];
-#pragma unroll
-      for (int j = 0; j < NT; ++j) {
-        float2 v = __fadd2_rn(U[j][3], sb);
-        v = __ffma2_rn(U[j][0], sx, v);
-        v = __ffma2_rn(U[j][1], sy, v);
-        v = __ffma2_rn(U[j][2], sz, v);
-        float2 rinv, phs;
-        if (MODE == 0) {
-          rinv = make_float2(rsqrt_ftz(v.x), rsqrt_ftz(v.y));
-          phs = __ffma2_rn(kap2, __fmul2_rn(v, rinv), nkr0);
-        } else {
-          const float2 r2 = __fadd2_rn(v, r0sq);
-          rinv = make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y));
-          const float2 den = __ffma2_rn(__fmul2_rn(r2, rinv), kinv2, r0k);
-          phs = __fmul2_rn(v, make_float2(rcp_ftz(den.x), rcp_ftz(den.y)));
-          if (MODE == 2) {
-            const float2 qq = __fmul2_rn(phs, make_float2(inv2pi, inv2pi));
-            const float2 qn = make_float2(-rintf(qq.x), -rintf(qq.y));
-            phs = __ffma2_rn(qn, make_float2(c1, c1), phs);
-            phs = __ffma2_rn(qn, make_float2(c2, c2), phs);
-          }
-        }
-        const float2 sn = make_float2(sin_ftz(phs.x), sin_ftz(phs.y));
-        const float2 cs = make_float2(cos_ftz(phs.x), cos_ftz(phs.y));
-        gr[j] = __fmul2_rn(cs, rinv);
-        gi[j] = __fmul2_rn(sn, rinv);
-      }
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const float4 fr = sF[6 * kp + h], fi = sF[6 * kp + 2 + h], fn = sF[6 * kp + 4 + h];
-#pragma unroll
-        for (int qq = 0; qq < 2; ++qq) {
-          const int q = 2 * h + qq;
-          const float2 wr = qq ? make_float2(fr.z, fr.w) : make_float2(fr.x, fr.y);
-          const float2 wi = qq ? make_float2(fi.z, fi.w) : make_float2(fi.x, fi.y);
-          const float2 wn = qq ? make_float2(fn.z, fn.w) : make_float2(fn.x, fn.y);
-#pragma unroll
-          for (int j = 0; j < NT; ++j) {
-            are[j][q] = __ffma2_rn(gi[j], wn, __ffma2_rn(gr[j], wr, are[j][q]));
-            aim[j][q] = __ffma2_rn(gi[j], wr, __ffma2_rn(gr[j], wi, aim[j][q]));
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < NT; ++j)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        float *h0 = sA + (j * 16 + 2 * q) * 32 + lane, *h1 = h0 + 32, *l0 = h0 + 8 * 32, *l1 = h1 + 8 * 32;
-        float vh0 = *h0, vl0 = *l0, vh1 = *h1, vl1 = *l1;
-        two_sum_acc(vh0, vl0, are[j][q].x + are[j][q].y);
-        two_sum_acc(vh1, vl1, aim[j][q].x + aim[j][q].y);
-        *h0 = vh0;
-        *l0 = vl0;
-        *h1 = vh1;
-        *l1 = vl1;
-      }
-  }
-#pragma unroll
-  for (int j = 0; j < NT; ++j) {
-    int mi = lane + j * T;
-    if (lane < T && mi < nI) {
-      float o[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) o[q] = sA[(j * 16 + q) * 32 + lane] + sA[(j * 16 + 8 + q) * 32 + lane];
-      acc[2 * ((size_t)t * nI + mi)] = make_float4(o[0], o[1], o[2], o[3]);
-      acc[2 * ((size_t)t * nI + mi) + 1] = make_float4(o[4], o[5], o[6], o[7]);
-    }
-  }
-}
-
-// FP32 M2L over unordered admissible pairs: every coupling tile K_ts (entries as in
-// k_m2l_f32w) is evaluated once and applied in both directions, acc_t += K_ts w_s and
-// acc_s += K_ts^T w_t (K is symmetric in the two clusters: it depends on |x_t - x_s| only).
 // One warp per owner cluster t; lane l < T owns the target rows m = l + j T (j < NT).  The
 // tile is swept along its diagonals: at step k lane l takes the source column c = (l + k) mod
 // nI, so the row sums stay in the lane (forward) and the column sum of column c moves one lane
@@ -714,13 +530,20 @@ __global__ void k_m2l_sym_reduce(int nred, const int *__restrict__ red, const in
   acc[2 * ((size_t)c * nI + m) + 1] = make_float4(h[4] + l[4], h[5] + l[5], h[6] + l[6], h[7] + l[7]);
 }
 
+// acc: `nslab` partial results of the M2L (splits of the source lists), `slab` float4 apart,
+// added in order
 __global__ void k_unfold_f32n(long long tot, int nI, float ik2, const double *__restrict__ nodeD,
-                              const float4 *__restrict__ acc, float2 *__restrict__ loc) {
+                              const float4 *__restrict__ acc, int nslab, size_t slab, float2 *__restrict__ loc) {
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= tot) return;
   int id = (int)(t / nI), mi = (int)(t % nI);
   const double *D = nodeD + 6 * t;
   float4 u = acc[2 * t], v = acc[2 * t + 1];
+  for (int k = 1; k < nslab; ++k) {
+    const float4 a = acc[k * slab + 2 * t], b = acc[k * slab + 2 * t + 1];
+    u = make_float4(u.x + a.x, u.y + a.y, u.z + a.z, u.w + a.w);
+    v = make_float4(v.x + b.x, v.y + b.y, v.z + b.z, v.w + b.w);
+  }
   float cr[3] = {u.x, u.z, v.x}, ci[3] = {u.y, u.w, v.y};
   float l0x = 0, l0y = 0, l1x = 0, l1y = 0;
   for (int k = 0; k < 3; ++k) {
@@ -1006,11 +829,6 @@ __global__ void k_leaf_eval(int nE, int leaf_off, int p1, int q1, R h, const dou
 // ------------------------------------------------------------------------ drivers
 constexpr int kM2LWarps = 4;
 
-// per warp: target nodes, staged source pairs, running sums [NT][16][32] (NT = ceil(nI / 32))
-static size_t m2l_f32_smem(int nI) {
-  return sizeof(float4) * ((size_t)nI + 8 * (size_t)((nI + 1) / 2) + 4 * 32 * (size_t)((nI + 31) / 32)) * kM2LWarps;
-}
-
 static size_t m2l_sym_smem(int nI) {
   return sizeof(float4) * (6 * (size_t)nI + 4 * 32 * (size_t)((nI + 31) / 32)) * kM2LWarps;
 }
@@ -1056,43 +874,18 @@ static efie_status launch_m2l_sym_t(Ctx *c, cudaStream_t st) {
   return EFIE_OK;
 }
 
-template <int MODE>
-static efie_status launch_m2l_f32_t(Ctx *c, cudaStream_t st) {
-  if (c->d_back) return launch_m2l_sym_t<MODE>(c, st);
-  const int nI = c->nI, NT = (nI + 31) / 32;
-  const unsigned blocks = (unsigned)((c->n_m2l_targets + kM2LWarps - 1) / kM2LWarps);
-  const size_t sm = m2l_f32_smem(nI);
-  const float kf = (float)c->kappa;
-  switch (NT) {
-#define EFIE_M2L_CASE(N)                                                                                      \
-  case N:                                                                                                    \
-    k_m2l_f32w<N, MODE><<<blocks, 32 * kM2LWarps, sm, st>>>(c->d_m2l_targets, c->n_m2l_targets, c->d_far_ptr,  \
-                                                           c->d_far_src, c->d_pgeo, c->d_pph, nI, kf,          \
-                                                           c->d_nodeX4, c->d_srcf, c->d_accf);                 \
-    ++c->launches;                                                                                           \
-    break;
-    EFIE_M2L_CASE(1)
-    EFIE_M2L_CASE(2)
-    EFIE_M2L_CASE(3)
-    EFIE_M2L_CASE(4)
-    EFIE_M2L_CASE(5)
-    EFIE_M2L_CASE(6)
-    EFIE_M2L_CASE(7)
-    EFIE_M2L_CASE(8)
-    EFIE_M2L_CASE(9)
-    EFIE_M2L_CASE(10)
-#undef EFIE_M2L_CASE
-    default:
-      c->err = "q too large for the FP32 M2L kernel";
-      return EFIE_EINVAL;
+// M2L of one right-hand side in the mixed form, d_srcf -> d_accf; *nslab partial results
+static efie_status launch_m2l_f32(Ctx *c, cudaStream_t st, int *nslab) {
+  *nslab = 1;
+  if (c->d_back) {
+    if (c->m2l_mode == 0) return launch_m2l_sym_t<0>(c, st);
+    if (c->m2l_mode == 1) return launch_m2l_sym_t<1>(c, st);
+    return launch_m2l_sym_t<2>(c, st);
   }
-  return EFIE_OK;
-}
-
-static efie_status launch_m2l_f32(Ctx *c, cudaStream_t st) {
-  if (c->m2l_mode == 0) return launch_m2l_f32_t<0>(c, st);
-  if (c->m2l_mode == 1) return launch_m2l_f32_t<1>(c, st);
-  return launch_m2l_f32_t<2>(c, st);
+  *nslab = c->m2l_split;
+  const size_t slab = (size_t)c->ncl * 4 * c->nI;
+  float2 *acc = reinterpret_cast<float2 *>(c->d_accf);
+  return launch_m2l_mma(c, st, {1, 4, c->m2l_split, reinterpret_cast<const float2 *>(c->d_srcf), acc, acc + slab, 4, slab});
 }
 
 static efie_status launch_m2l_stored(Ctx *c, cudaStream_t st, bool f32) {
@@ -1186,25 +979,14 @@ static efie_status m2l_sym_attrs(int bytes) {
   return e == cudaSuccess ? EFIE_OK : EFIE_ECUDA;
 }
 
-template <int MODE>
-static efie_status m2l_f32_attrs(int bytes) {
-  cudaError_t e = cudaSuccess;
-  for (auto f : {k_m2l_f32w<1, MODE>, k_m2l_f32w<2, MODE>, k_m2l_f32w<3, MODE>, k_m2l_f32w<4, MODE>,
-                 k_m2l_f32w<5, MODE>, k_m2l_f32w<6, MODE>, k_m2l_f32w<7, MODE>, k_m2l_f32w<8, MODE>,
-                 k_m2l_f32w<9, MODE>, k_m2l_f32w<10, MODE>})
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  return e == cudaSuccess ? EFIE_OK : EFIE_ECUDA;
-}
-
-static efie_status launch_m2l_f32(Ctx *c, cudaStream_t st);
-
 // Best of 3 device times (CUDA events on the context stream) of the M2L as it is configured.
 static efie_status time_m2l(Ctx *c, float *best) {
-  EFIE_TRY(launch_m2l_f32(c, c->stream));  // warm-up
+  int nslab = 1;
+  EFIE_TRY(launch_m2l_f32(c, c->stream, &nslab));  // warm-up
   *best = 1e30f;
   for (int r = 0; r < 3; ++r) {
     EFIE_CUDA(cudaEventRecord(c->tm.ev[3], c->stream));
-    EFIE_TRY(launch_m2l_f32(c, c->stream));
+    EFIE_TRY(launch_m2l_f32(c, c->stream, &nslab));
     EFIE_CUDA(cudaEventRecord(c->tm.ev[4], c->stream));
     EFIE_CUDA(cudaEventSynchronize(c->tm.ev[4]));
     float ms = 0.f;
@@ -1214,8 +996,7 @@ static efie_status time_m2l(Ctx *c, float *best) {
   return EFIE_OK;
 }
 
-// M2L autotuner (option m2l_pairs = 2): the ordered-pair kernel (one warp per target cluster,
-// its whole far list) and the unordered-pair kernel (one warp per owner, each coupling tile
+// M2L autotuner (option m2l_pairs = 2): the ordered-pair kernel (a block per target cluster) and the unordered-pair kernel (one warp per owner, each coupling tile
 // applied both ways) are timed on this problem's blocks and the faster is kept; the other's
 // buffers are returned.  Sources are zero during the timing (the work does not depend on them).
 static efie_status m2l_autotune(Ctx *c) {
@@ -1235,7 +1016,7 @@ static efie_status m2l_autotune(Ctx *c) {
     dfree(c, c->d_own_pgeo);
     dfree(c, c->d_own_pph);
   }
-  EFIE_CUDA(cudaMemsetAsync(c->d_accf, 0, sizeof(float4) * (size_t)c->ncl * 2 * c->nI, c->stream));
+  EFIE_CUDA(cudaMemsetAsync(c->d_accf, 0, sizeof(float4) * (size_t)c->m2l_split * c->ncl * 2 * c->nI, c->stream));
   EFIE_CUDA(cudaStreamSynchronize(c->stream));
   return EFIE_OK;
 }
@@ -1260,9 +1041,6 @@ static efie_status m2l_f32_tables(Ctx *c) {
     ++c->launches;
     EFIE_CUDA(cudaGetLastError());
   }
-  EFIE_TRY(m2l_f32_attrs<0>((int)m2l_f32_smem(kMaxQ1 * kMaxQ1)));
-  EFIE_TRY(m2l_f32_attrs<1>((int)m2l_f32_smem(kMaxQ1 * kMaxQ1)));
-  EFIE_TRY(m2l_f32_attrs<2>((int)m2l_f32_smem(kMaxQ1 * kMaxQ1)));
   // unordered-pair form (option m2l_pairs): the column sums of every pair take npairs x nI x 32
   // bytes; used when they fit in a quarter of the free memory, else the one-sided kernel runs
   dfree(c, c->d_back);
@@ -1311,6 +1089,7 @@ static efie_status far_chain(Ctx *c, const double2 *xs, double2 *ys, C2<R> *mom,
     k_fold_f32n<<<gtot, 256, 0, st>>>(tot, nI, c->d_nodeD, (const float2 *)mom, c->d_srcf); ++c->launches;
   }
   cudaEventRecord(c->tm.ev[3], st);
+  int nslab = 1;
   if (c->n_m2l_targets > 0 && c->k_stored) {
     EFIE_TRY(launch_m2l_stored(c, st, sizeof(R) == 4));
   } else if (c->n_m2l_targets > 0) {
@@ -1320,7 +1099,7 @@ static efie_status far_chain(Ctx *c, const double2 *xs, double2 *ys, C2<R> *mom,
       k_m2l_f64<<<c->n_m2l_targets, thr, sm, st>>>(c->d_m2l_targets, c->d_far_ptr, c->d_far_src, nI, c->kappa,
                                                    c->d_nodeX, (const double2 *)srcv, c->d_acc); ++c->launches;
     } else {
-      EFIE_TRY(launch_m2l_f32(c, st));
+      EFIE_TRY(launch_m2l_f32(c, st, &nslab));
     }
   }
   cudaEventRecord(c->tm.ev[4], st);
@@ -1329,7 +1108,7 @@ static efie_status far_chain(Ctx *c, const double2 *xs, double2 *ys, C2<R> *mom,
                                                     (double2 *)loc); ++c->launches;
   } else {
     k_unfold_f32n<<<gtot, 256, 0, st>>>(tot, nI, (float)(1.0 / (c->kappa * c->kappa)), c->d_nodeD, c->d_accf,
-                                        (float2 *)loc); ++c->launches;
+                                        nslab, (size_t)c->ncl * 2 * nI, (float2 *)loc); ++c->launches;
   }
   for (int l = 0; l < m; ++l) {
     int npar = c->np << (2 * l);
@@ -1418,8 +1197,10 @@ efie_status dev_alloc_work(Ctx *c) {
   if (c->opt.precision == EFIE_MIXED_FP32) {
     EFIE_TRY(dalloc(c, &c->d_momf, ncl * 3 * nI));
     EFIE_TRY(dalloc(c, &c->d_srcf, ncl * 2 * nI));
-    EFIE_TRY(dalloc(c, &c->d_accf, ncl * 2 * nI));
-    EFIE_CUDA(cudaMemsetAsync(c->d_accf, 0, sizeof(float4) * ncl * 2 * nI, c->stream));
+    c->m2l_split = m2l_mma_splits(c);
+    const size_t slabs = (size_t)c->m2l_split * ncl * 2 * nI;
+    EFIE_TRY(dalloc(c, &c->d_accf, slabs));
+    EFIE_CUDA(cudaMemsetAsync(c->d_accf, 0, sizeof(float4) * slabs, c->stream));
     EFIE_TRY(dalloc(c, &c->d_locf, ncl * 3 * nI));
     EFIE_TRY(m2l_f32_tables(c));
   } else {
@@ -1442,8 +1223,9 @@ efie_status dev_alloc_work(Ctx *c) {
 
 // ========================================================================================
 // Several right-hand sides at once (mixed form).  The cheap stages run once per right-hand
-// side; the M2L evaluates the coupling tile G(m, m') of every admissible block once into
-// shared memory and applies it to the 4 fields of up to kRB right-hand sides.
+// side; the M2L applies the coupling of every admissible block to the fields of many right-hand
+// sides (m2l_mma.cu for a few, m2l_tc.cu for many; option m2l_batch = 1: k_m2l_f32_multi, which
+// evaluates the coupling tile once into shared memory for up to kRB right-hand sides).
 namespace efie {
 
 constexpr int kRB = 8;             // right-hand sides per M2L block
@@ -1474,14 +1256,21 @@ __global__ void k_fold_multi(long long tot, int nI, int R, int ld, size_t mstrid
 }
 
 __global__ void k_unfold_multi(long long tot, int nI, int R, int ld, size_t lstride, float ik2,
-                               const double *__restrict__ nodeD,
-                               const float2 *__restrict__ acc, float2 *__restrict__ loc) {
+                               const double *__restrict__ nodeD, const float2 *__restrict__ acc,
+                               const float2 *__restrict__ more, int nslab, size_t slab, float2 *__restrict__ loc) {
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= tot) return;
   const int id = (int)(t / nI), mi = (int)(t % nI);
   const double *D = nodeD + 6 * t;
   for (int r = 0; r < R; ++r) {
-    const float2 *a = acc + (size_t)t * ld + 4 * r;
+    float2 a[4];
+    for (int k = 0; k < 4; ++k) {
+      a[k] = acc[(size_t)t * ld + 4 * r + k];
+      for (int j = 1; j < nslab; ++j) {
+        const float2 b = more[(j - 1) * slab + (size_t)t * (4 * kMmaMaxRhs) + 4 * r + k];
+        a[k] = make_float2(a[k].x + b.x, a[k].y + b.y);
+      }
+    }
     float l0x = 0, l0y = 0, l1x = 0, l1y = 0;
     for (int k = 0; k < 3; ++k) {
       l0x += (float)D[k] * a[k].x;
@@ -1604,6 +1393,11 @@ efie_status dev_batch_alloc(Ctx *c, int R) {
   EFIE_TRY(dalloc(c, &c->d_srcB, (size_t)R * ncl * 4 * nI));
   EFIE_TRY(dalloc(c, &c->d_accB, (size_t)R * ncl * 4 * nI));
   EFIE_CUDA(cudaMemsetAsync(c->d_accB, 0, sizeof(float2) * (size_t)R * ncl * 4 * nI, c->stream));
+  if (c->m2l_split > 1 && !c->d_moreB) {
+    const size_t more = (size_t)(c->m2l_split - 1) * ncl * nI * 4 * kMmaMaxRhs;
+    EFIE_TRY(dalloc(c, &c->d_moreB, more));
+    EFIE_CUDA(cudaMemsetAsync(c->d_moreB, 0, sizeof(float2) * more, c->stream));
+  }
   EFIE_TRY(dalloc(c, &c->d_locB, (size_t)R * ncl * 3 * nI));
   if (c->opt.precision == EFIE_MIXED_FP32 && m2l_tc_supported(c)) EFIE_TRY(m2l_tc_prepare(c));
   const int sm = (int)multi_smem(kMultiMaxNI);
@@ -1622,7 +1416,7 @@ __global__ void k_sum2(size_t n, const double2 *__restrict__ a, const double2 *_
 // Y[r] = A X[r], r < R (host arrays of device pointers).  superspace: X[r] and Y[r] are
 // superspace vectors and the product is (N + F) X[r] (no T gather / scatter).
 efie_status dev_matvec_batch(Ctx *c, int R, const double2 *const *X, double2 *const *Y, bool superspace) {
-  if (c->opt.precision != EFIE_MIXED_FP32 || R == 1 || (c->nI > kMultiMaxNI && !m2l_tc_supported(c))) {
+  if (c->opt.precision != EFIE_MIXED_FP32 || R == 1 || (c->opt.m2l_batch == 1 && c->nI > kMultiMaxNI)) {
     for (int r = 0; r < R; ++r) EFIE_TRY(superspace ? dev_matvec_super(c, X[r], Y[r]) : dev_matvec(c, X[r], Y[r]));
     return EFIE_OK;
   }
@@ -1662,8 +1456,14 @@ efie_status dev_matvec_batch(Ctx *c, int R, const double2 *const *X, double2 *co
   const int ld = 4 * c->batch_cap;
   k_fold_multi<<<gtot, 256, 0, st>>>(tot, nI, R, ld, mstride, c->d_nodeD, c->d_momB, c->d_srcB); ++c->launches;
   EFIE_CUDA(cudaEventRecord(c->tm.ev[3], st));
-  const bool use_tc = c->opt.m2l_batch != 1 && m2l_tc_supported(c);
-  if (c->n_m2l_targets > 0 && use_tc) {
+  // a few right-hand sides, or tiles too large for tensor memory: kernel entries in mma.sync operands
+  const bool use_mma = c->opt.m2l_batch != 1 && R <= m2l_mma_rhs(c);
+  const bool use_tc = c->opt.m2l_batch != 1 && !use_mma;
+  const int nslab = use_mma && R <= kMmaMaxRhs ? c->m2l_split : 1;
+  const size_t slab = (size_t)c->ncl * nI * 4 * kMmaMaxRhs;
+  if (c->n_m2l_targets > 0 && use_mma) {
+    EFIE_TRY(launch_m2l_mma(c, st, {R, ld, nslab, c->d_srcB, c->d_accB, c->d_moreB, 4 * kMmaMaxRhs, slab}));
+  } else if (c->n_m2l_targets > 0 && use_tc) {
     EFIE_TRY(launch_m2l_tc(c, st, 4 * R, ld, c->d_srcB, c->d_accB));
   } else if (c->n_m2l_targets > 0) {
     const int F = 4 * R, KM = (nI + 7) / 8;
@@ -1686,7 +1486,7 @@ efie_status dev_matvec_batch(Ctx *c, int R, const double2 *const *X, double2 *co
   }
   EFIE_CUDA(cudaEventRecord(c->tm.ev[4], st));
   k_unfold_multi<<<gtot, 256, 0, st>>>(tot, nI, R, ld, mstride, (float)(1.0 / (c->kappa * c->kappa)), c->d_nodeD,
-                                       c->d_accB, c->d_locB); ++c->launches;
+                                       c->d_accB, c->d_moreB, nslab, slab, c->d_locB); ++c->launches;
   for (int l = 0; l < m; ++l) {
     int npar = c->np << (2 * l);
     k_l2l<float><<<dim3(npar, R), 128, l2l_smem(q1, sizeof(float2)), st>>>(npar, c->lev_off[l], c->lev_off[l + 1], q1,

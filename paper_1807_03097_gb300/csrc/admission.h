@@ -41,11 +41,14 @@ inline size_t request_footprint(int np, int level_m, int p, int q, int gmres_res
   const size_t batch = lockstep > 1 ? lockstep * (5 * nE * nb * 16 + 14 * ncl * nI * 8 + 4 * ndof * 16) : 0;
   const size_t farfield = ndir > 0 ? 48 * size_t(ndir) * nE + 48 * size_t(ndir) + 24 * size_t(ndir) : 0;
   const bool stored = mixed ? m2l_store == 2 : m2l_store != 1;
-  const size_t coupling = stored ? 130 * ncl * nI * nI * (mixed ? 8 : 16) : 0;
+  // FP64: rows in tiles of 16, an even number of columns
+  const size_t entries = mixed ? nI * nI : (nI + 15) / 16 * 16 * ((nI + 1) / 2 * 2);
+  const size_t coupling = stored ? 130 * ncl * entries * (mixed ? 8 : 16) : 0;
   // partial M2L results of small problems, whose source lists are split over blocks (at most 16
   // splits, of few enough clusters that splits x clusters stays near 2 x 8 blocks per SM)
+  const size_t fix64 = !mixed && stored ? ncl * nI * 64 + std::min<size_t>(15 * ncl, 9728) * nI * 64 : 0;
   const size_t splits = mixed ? std::min<size_t>(15 * ncl, 4864) * nI * (32 + (lockstep > 1 ? 256 : 0)) : 0;
-  return near + krylov + clusters + vecs + batch + farfield + coupling + splits + (size_t(64) << 20);
+  return near + krylov + clusters + vecs + batch + farfield + coupling + splits + fix64 + (size_t(64) << 20);
 }
 
 inline int pick_admission(int nqueued, const size_t *footprint, const double *cost, int oldest_passed, size_t left,

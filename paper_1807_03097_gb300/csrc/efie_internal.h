@@ -120,6 +120,13 @@ struct Ctx {
   float m2l_tune_ms[2] = {0.f, 0.f};  // autotuned M2L (m2l_pairs = 2): ordered, unordered
   void *d_K = nullptr;        // stored coupling matrices [pair][m'][m] (double2 or float2)
   bool k_stored = false;
+  // FP64 form: kept matrices as digits for the FP16 tensor cores (m2l_f64.cu)
+  bool k_digits = false;
+  size_t *d_koff = nullptr;   // [ncl + 1] K-steps before every cluster's matrices
+  int *d_kexp = nullptr;      // [ncl] fixed-point exponent of a target's matrices
+  unsigned long long *d_smax = nullptr, *d_fix = nullptr;  // largest source per level and field; fixed-point sources
+  double2 *d_accmore = nullptr;  // [f64_split - 1][ncl][4][nI]: further splits of d_acc
+  int f64_split = 1;
   // several right-hand sides (mixed form)
   int batch_cap = 0;
   double *h_resB = nullptr;  // pinned residual estimates of a lockstep batch
@@ -237,6 +244,11 @@ struct MmaArgs {
 int m2l_mma_splits(const Ctx *c);
 int m2l_mma_rhs(const Ctx *c);  // right-hand sides up to which a batch takes it
 efie_status launch_m2l_mma(Ctx *c, cudaStream_t st, const MmaArgs &A);
+// FP64 M2L from kept matrices in digits on the FP16 tensor cores (m2l_f64.cu)
+size_t m2l_f64_digits_bytes(const Ctx *c);
+efie_status m2l_f64_digits_build(Ctx *c);
+efie_status m2l_f64_digits_fold(Ctx *c, cudaStream_t st, const double2 *mom, double2 *src);
+efie_status m2l_f64_digits_apply(Ctx *c, cudaStream_t st);
 // tensor-core M2L of a batch (m2l_tc.cu)
 bool m2l_tc_supported(const Ctx *c);
 efie_status m2l_tc_prepare(Ctx *c);

@@ -192,17 +192,27 @@ __global__ void k_fold(long long tot, int nI, const double *__restrict__ nodeD, 
   s[3 * nI + mi] = mm[2 * nI + mi];
 }
 
+// acc plus nslab - 1 further partial results of the M2L in `more` (splits of the source lists)
 template <class R, class A>
 __global__ void k_unfold(long long tot, int nI, R ik2, const double *__restrict__ nodeD, const A *__restrict__ acc,
-                         C2<R> *__restrict__ loc) {
+                         const A *__restrict__ more, int nslab, size_t slab, C2<R> *__restrict__ loc) {
   long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= tot) return;
   int id = (int)(t / nI), mi = (int)(t % nI);
   const double *D = nodeD + 6 * t;
-  const A *a = acc + (size_t)id * 4 * nI;
+  A sum[4];
+  for (int k = 0; k < 4; ++k) {
+    const size_t at = ((size_t)id * 4 + k) * nI + mi;
+    sum[k] = acc[at];
+    for (int j = 1; j < nslab; ++j) {
+      const A b = more[(j - 1) * slab + at];
+      sum[k].x += b.x;
+      sum[k].y += b.y;
+    }
+  }
   R l0x = 0, l0y = 0, l1x = 0, l1y = 0;
   for (int k = 0; k < 3; ++k) {
-    A v = a[k * nI + mi];
+    A v = sum[k];
     l0x += (R)D[k] * (R)v.x;
     l0y += (R)D[k] * (R)v.y;
     l1x += (R)D[3 + k] * (R)v.x;
@@ -211,7 +221,7 @@ __global__ void k_unfold(long long tot, int nI, R ik2, const double *__restrict_
   C2<R> *l = loc + (size_t)id * 3 * nI;
   l[mi] = mk<R>(l0x, l0y);
   l[nI + mi] = mk<R>(l1x, l1y);
-  A dv = a[3 * nI + mi];
+  A dv = sum[3];
   l[2 * nI + mi] = mk<R>(-ik2 * (R)dv.x, -ik2 * (R)dv.y);
 }
 
@@ -926,7 +936,7 @@ static efie_status launch_m2l_stored(Ctx *c, cudaStream_t st, bool f32) {
 // Decide whether the coupling matrices are kept (m2l_store option) and evaluate them.
 static efie_status m2l_store_matrices(Ctx *c) {
   dfree(c, c->d_K);
-  c->k_stored = false;
+  c->k_stored = c->k_digits = false;
   if (c->nfar == 0 || c->opt.m2l_store == 1) return EFIE_OK;
   const bool f32 = c->opt.precision == EFIE_MIXED_FP32;
   const size_t nI2 = (size_t)c->nI * c->nI;
@@ -936,7 +946,19 @@ static efie_status m2l_store_matrices(Ctx *c) {
   // auto: keep them for the FP64 form only (evaluating FP64 sine / cosine / sqrt is the
   // bottleneck of that form on this GPU, while the FP32 form evaluates faster than HBM can
   // stream the stored matrices)
-  if (c->opt.m2l_store == 0 && (f32 || bytes > freeb / 2)) return EFIE_OK;
+  if (c->opt.m2l_store == 0 && f32) return EFIE_OK;
+  // FP64 form: as digits for the tensor cores (rows padded to 16 target nodes, so 1.2 to 1.3 times the
+  // bytes at q >= 4), else, where only the plain matrices fit, for the FP64 pipe
+  if (!f32 && 2 * c->npairs == c->nfar) {
+    const size_t digits = m2l_f64_digits_bytes(c);
+    if (digits <= (c->opt.m2l_store == 0 ? freeb / 2 : freeb) && pool_alloc(c, &c->d_K, digits) == EFIE_OK) {
+      EFIE_TRY(m2l_f64_digits_build(c));
+      c->k_stored = c->k_digits = true;
+      return EFIE_OK;
+    }
+    c->d_K = nullptr;
+  }
+  if (c->opt.m2l_store == 0 && bytes > freeb / 2) return EFIE_OK;
   if (pool_alloc(c, &c->d_K, bytes) != EFIE_OK) {
     c->d_K = nullptr;
     if (c->opt.m2l_store == 2) {
@@ -1083,14 +1105,19 @@ static efie_status far_chain(Ctx *c, const double2 *xs, double2 *ys, C2<R> *mom,
   }
   long long tot = (long long)c->ncl * nI;
   const unsigned gtot = (unsigned)((tot + 255) / 256);
-  if (sizeof(R) == 8) {
+  if (sizeof(R) == 8 && c->k_digits) {
+    EFIE_TRY(m2l_f64_digits_fold(c, st, (const double2 *)mom, (double2 *)srcv));
+  } else if (sizeof(R) == 8) {
     k_fold<double><<<gtot, 256, 0, st>>>(tot, nI, c->d_nodeD, (const double2 *)mom, (double2 *)srcv); ++c->launches;
   } else {
     k_fold_f32n<<<gtot, 256, 0, st>>>(tot, nI, c->d_nodeD, (const float2 *)mom, c->d_srcf); ++c->launches;
   }
   cudaEventRecord(c->tm.ev[3], st);
   int nslab = 1;
-  if (c->n_m2l_targets > 0 && c->k_stored) {
+  if (c->n_m2l_targets > 0 && c->k_digits) {
+    EFIE_TRY(m2l_f64_digits_apply(c, st));
+    nslab = c->f64_split;
+  } else if (c->n_m2l_targets > 0 && c->k_stored) {
     EFIE_TRY(launch_m2l_stored(c, st, sizeof(R) == 4));
   } else if (c->n_m2l_targets > 0) {
     if (sizeof(R) == 8) {
@@ -1105,7 +1132,8 @@ static efie_status far_chain(Ctx *c, const double2 *xs, double2 *ys, C2<R> *mom,
   cudaEventRecord(c->tm.ev[4], st);
   if (sizeof(R) == 8) {
     k_unfold<double, double2><<<gtot, 256, 0, st>>>(tot, nI, 1.0 / (c->kappa * c->kappa), c->d_nodeD, c->d_acc,
-                                                    (double2 *)loc); ++c->launches;
+                                                    c->d_accmore, nslab, (size_t)c->ncl * 4 * nI, (double2 *)loc);
+    ++c->launches;
   } else {
     k_unfold_f32n<<<gtot, 256, 0, st>>>(tot, nI, (float)(1.0 / (c->kappa * c->kappa)), c->d_nodeD, c->d_accf,
                                         nslab, (size_t)c->ncl * 2 * nI, (float2 *)loc); ++c->launches;

@@ -1,0 +1,434 @@
+// M2L of the FP64 form with kept coupling matrices (a6, Sec. 4.2: acc_t(f, i) = sum_s sum_j
+// G(x_ti, x_sj) u_s(f, j)), as exact integer products on the FP16 tensor cores.
+//
+// Why: GB300 issues one FP64 FMA warp instruction per 72 clocks and scheduler, so the 16 FMAs of an
+// entry (4 complex fields) bound the product at 22 times the time that HBM needs to deliver the
+// matrices.  Here every matrix entry and every folded source field is a fixed-point number of
+// six 10-bit digits.  A digit is exact in FP16, a product of two digits has at most 18 bits, and
+// the tensor core's FP32 accumulators hold the sums of 16 nodes (real and imaginary part)
+// exactly; they go into 64-bit integers, which are rounded to FP64 once per target node.
+//
+// Fixed point.  w = rint(v 2^(58 - e)) with 2^e above the largest |Re|, |Im| (matrices: per target
+// cluster, from the smallest node distance of its far list; sources: per tree level and field,
+// found in every product); u = w + O, O = sum_k 512 1024^k, has the unsigned digits d_k, so that
+// w = sum_k c_k 1024^k with c_k = d_k - 512 in [-512, 511] (the leading one in [-257, 256]).
+// Digit products are summed by total weight: diagonal D holds c_k c'_l with (5 - k) + (5 - l) = D,
+// D <= 5 (21 of 36 products; the rest is below 2^-57 of the largest product).  Sums over 16 nodes
+// x 2 parts stay below 2^24 for D <= 3 (D = 3 in two accumulators), hence exact; a rounding of D = 4, 5
+// is below 2^-58.  The product differs from the one with evaluated FP64 entries by 5.9e-16 (relative
+// 2-norm, sphere of 1 536 elements, 81 nodes; the FP64 pipe's sums over kept matrices by 8.0e-16).
+//
+// Bound: HBM delivers the words (two FP64 a complex entry, rows padded to 16); beside it a
+// scheduler spends about 64 clocks per 32 entries on products and digits.  Measured, M2L before (FP64 pipe,
+// kept matrices) and after: 52.7 -> 3.5 ms at 125 760 pairs of 81 nodes (15.1 GB, 4.5 TB/s of 6.7), 163 -> 8.2 ms
+// at 121 nodes, 6.95 -> 0.36 ms at 49, 1.55 -> 0.034 ms at 5 472 pairs of 25 (few targets: the K-steps
+// of a target are split over blocks), 0.26 -> 0.041 ms at 4 nodes, where 12 of 16 rows are padding.
+//
+// Layout of the kept matrices: per target cluster, 16 source nodes (a K-step) x 16 target
+// nodes (a row tile) at a time, the words of one A fragment of mma.m16n8k16 per lane.  A fragment
+// register is a pair of entries (source nodes 2 q, 2 q + 1 of one row); its 2 x 6 digits take four
+// 32-bit words: the low 10 bits of each half are the digits 5, 4, 3, 2, the high 6 bits hold digits
+// 1 and 0 in pieces (6 + 4 bits).  So an entry keeps its 16 bytes, a warp reads 512 contiguous
+// bytes per load, and a digit becomes FP16 by one mask-and-or (0x6400 | d is 1024 + d) and one
+// packed subtraction (two more shifts for digits 1, 0).
+#include <algorithm>
+#include <cmath>
+#include <cuda_fp16.h>
+
+#include "efie_internal.h"
+
+namespace efie {
+
+namespace {
+
+constexpr unsigned long long kOffset = 512ull * 0x0004010040100401ull;  // 512 sum_k 2^(10 k), k < 6
+constexpr int kFixBits = 58;
+constexpr int kF64Nodes = 64;  // source nodes staged at a time
+
+struct LevOff {
+  int off[12];
+};
+
+__device__ __forceinline__ int level_of(const LevOff &L, int m, int id) {
+  int l = 0;
+  while (l < m && id >= L.off[l + 1]) ++l;
+  return l;
+}
+
+__device__ __forceinline__ unsigned long long fix(double v, int e) {
+  return (unsigned long long)__double2ll_rn(scalbn(v, kFixBits - e)) + kOffset;
+}
+
+// four words of a pair of entries (x in the low halves)
+__device__ __forceinline__ uint4 pack_pair(unsigned long long x, unsigned long long y) {
+  auto half4 = [](unsigned long long u, unsigned *h) {
+    const unsigned d0 = u & 1023, d1 = (u >> 10) & 1023;
+    h[0] = (unsigned)((u >> 50) & 1023) | ((d1 >> 4) << 10);
+    h[1] = (unsigned)((u >> 40) & 1023) | ((d1 & 15) << 12);
+    h[2] = (unsigned)((u >> 30) & 1023) | ((d0 >> 4) << 10);
+    h[3] = (unsigned)((u >> 20) & 1023) | ((d0 & 15) << 12);
+  };
+  unsigned a[4], b[4];
+  half4(x, a);
+  half4(y, b);
+  return make_uint4(a[0] | (b[0] << 16), a[1] | (b[1] << 16), a[2] | (b[2] << 16), a[3] | (b[3] << 16));
+}
+
+// digit K (5 leading) of a pair as FP16 c_K
+template <int K>
+__device__ __forceinline__ unsigned digit(const uint4 &w) {
+  unsigned d;
+  if (K == 5) d = (w.x & 0x03ff03ffu) | 0x64006400u;
+  if (K == 4) d = (w.y & 0x03ff03ffu) | 0x64006400u;
+  if (K == 3) d = (w.z & 0x03ff03ffu) | 0x64006400u;
+  if (K == 2) d = (w.w & 0x03ff03ffu) | 0x64006400u;
+  if (K == 1) d = ((w.x >> 6) & 0x03f003f0u) | (((w.y >> 12) & 0x000f000fu) | 0x64006400u);
+  if (K == 0) d = ((w.z >> 6) & 0x03f003f0u) | (((w.w >> 12) & 0x000f000fu) | 0x64006400u);
+  const __half2 h = __hsub2(*reinterpret_cast<__half2 *>(&d), __float2half2_rn(1536.f));
+  return *reinterpret_cast<const unsigned *>(&h);
+}
+
+__device__ __forceinline__ void mma_f16(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+__device__ __forceinline__ uint4 ld_stream(const uint4 *p) {
+  uint4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+
+// products of digit K of the entries with the digits of the sources, b[2 l], b[2 l + 1] = digit 5 - l
+template <int K>
+__device__ __forceinline__ void digit_products(float (&D)[7][4], const uint4 (&w)[4], const unsigned (&b)[12]) {
+  const unsigned a[4] = {digit<K>(w[0]), digit<K>(w[1]), digit<K>(w[2]), digit<K>(w[3])};
+#pragma unroll
+  for (int l = 0; l <= K; ++l) {
+    const int d = (5 - K) + l;
+    // D = 3 in two accumulators (index 3: products with a leading digit, 6: the others)
+    mma_f16(D[d == 3 && K != 5 && l != 0 ? 6 : d], a, b[2 * l], b[2 * l + 1]);
+  }
+}
+
+}  // namespace
+
+// exponent e with 2^e >= 1.001 / (4 pi r) for every node distance r of a target's far list (distances
+// in FP32 from offsets to the cluster centres)
+__global__ void k_K_exponent(const int *__restrict__ targets, const int *__restrict__ fptr, const int *__restrict__ fsrc,
+                             int nI, const double *__restrict__ center, const float *__restrict__ nodeXf,
+                             int *__restrict__ expo) {
+  __shared__ float red[128];
+  const int t = targets[blockIdx.x];
+  float lo = 3e38f;
+  for (int k = fptr[t]; k < fptr[t + 1]; ++k) {
+    const int s = fsrc[k];
+    const float d0 = (float)(center[4 * t] - center[4 * s]), d1 = (float)(center[4 * t + 1] - center[4 * s + 1]),
+                d2 = (float)(center[4 * t + 2] - center[4 * s + 2]);
+    for (int i = threadIdx.x; i < nI * nI; i += blockDim.x) {
+      const float *a = nodeXf + ((size_t)t * nI + i / nI) * 3, *b = nodeXf + ((size_t)s * nI + i % nI) * 3;
+      const float x = d0 + a[0] - b[0], y = d1 + a[1] - b[1], z = d2 + a[2] - b[2];
+      lo = fminf(lo, x * x + y * y + z * z);
+    }
+  }
+  red[threadIdx.x] = lo;
+  __syncthreads();
+  for (int s = 64; s > 0; s >>= 1) {
+    if ((int)threadIdx.x < s) red[threadIdx.x] = fminf(red[threadIdx.x], red[threadIdx.x + s]);
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) expo[t] = ilogb(1.001 * 0.25 / (M_PI * sqrt((double)red[0]))) + 1;
+}
+
+// One block per unordered admissible pair {t, s}: G is symmetric, so every entry is evaluated once
+// and written into both clusters' matrices.  A thread owns 2 x 2 entries (nodes 2 a, 2 a + 1 of t, 2 b,
+// 2 b + 1 of s; the node count padded to an even nIe), i.e. two fragment words of either side.
+__global__ void __launch_bounds__(128) k_K_digits(int ncl, const int *__restrict__ optr, const int *__restrict__ osrc,
+                                                  const int *__restrict__ fptr, const int *__restrict__ fsrc,
+                                                  const size_t *__restrict__ koff, const int *__restrict__ expo, int nI,
+                                                  double kappa, const double *__restrict__ nodeX, uint4 *__restrict__ K) {
+  extern __shared__ double sx[];  // [2][nI][3]
+  __shared__ int sh[4];
+  const int u = blockIdx.x, tid = threadIdx.x;
+  if (tid == 0) {
+    int lo = 0, hi = ncl;  // the owner: optr[lo] <= u < optr[lo + 1]
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (optr[mid] <= u) lo = mid; else hi = mid;
+    }
+    sh[0] = lo;
+    sh[1] = osrc[u];
+  }
+  __syncthreads();
+  const int cl[2] = {sh[0], sh[1]};
+  for (int side = 0; side < 2; ++side)
+    for (int k = fptr[cl[side]] + tid; k < fptr[cl[side] + 1]; k += blockDim.x)
+      if (fsrc[k] == cl[1 - side]) sh[2 + side] = k - fptr[cl[side]];
+  for (int i = tid; i < 6 * nI; i += blockDim.x) sx[i] = nodeX[(size_t)cl[i / (3 * nI)] * 3 * nI + i % (3 * nI)];
+  __syncthreads();
+  const int nIe = (nI + 1) & ~1, nP = nIe >> 1, ntile = (nI + 15) >> 4;
+  const int e0 = expo[cl[0]], e1 = expo[cl[1]];
+  for (int idx = tid; idx < nP * nP; idx += blockDim.x) {
+    const int a = idx / nP, b = idx % nP;
+    double g[2][2][2];  // [node of t][node of s][re, im]
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const double *x = sx + 3 * min(2 * a + i, nI - 1), *y = sx + 3 * (nI + min(2 * b + j, nI - 1));
+        const double dx = x[0] - y[0], dy = x[1] - y[1], dz = x[2] - y[2];
+        const double r = sqrt(dx * dx + dy * dy + dz * dz);
+        double sn, cs;
+        sincos(kappa * r, &sn, &cs);
+        const double f = 0.25 / (M_PI * r);
+        g[i][j][0] = f * cs;
+        g[i][j][1] = f * sn;
+      }
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+      const int e = side == 0 ? e0 : e1;
+      const int J = sh[2 + side] * nIe + 2 * (side == 0 ? b : a), kk = J & 15;
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int row = 2 * (side == 0 ? a : b) + i;
+        if (row >= nI) continue;
+        const int lane = 4 * (row & 7) + ((kk & 7) >> 1), reg = ((row >> 3) & 1) + 2 * (kk >> 3);
+        uint4 *o = K + (((koff[cl[side]] + (J >> 4)) * ntile + (row >> 4)) * 8 + reg) * 32 + lane;
+#pragma unroll
+        for (int part = 0; part < 2; ++part) {
+          const double x = side == 0 ? g[i][0][part] : g[0][i][part], y = side == 0 ? g[i][1][part] : g[1][i][part];
+          __stcs(o + part * 128, pack_pair(fix(x, e), fix(y, e)));
+        }
+      }
+    }
+  }
+}
+
+// Folded source fields (as k_fold) and the largest |Re|, |Im| of each field on every level (bit
+// patterns of non-negative doubles order as integers; infinities and NaN come out above all).
+__global__ void k_fold_max(int nI, int m, LevOff L, const double *__restrict__ nodeD, const double2 *__restrict__ mom,
+                           double2 *__restrict__ src, unsigned long long *__restrict__ smax) {
+  __shared__ unsigned long long red[4][4];
+  const int id = blockIdx.x;
+  const double2 *mm = mom + (size_t)id * 3 * nI;
+  double2 *s = src + (size_t)id * 4 * nI;
+  unsigned long long big[4] = {0, 0, 0, 0};
+  auto note = [&](int f, double2 v) {
+    const unsigned long long a = __double_as_longlong(fabs(v.x)), b = __double_as_longlong(fabs(v.y));
+    big[f] = max(big[f], max(a, b));
+  };
+  for (int i = threadIdx.x; i < nI; i += blockDim.x) {
+    const double *D = nodeD + 6 * ((size_t)id * nI + i);
+    const double2 m0 = mm[i], m1 = mm[nI + i], nu = mm[2 * nI + i];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const double2 v = make_double2(D[k] * m0.x + D[3 + k] * m1.x, D[k] * m0.y + D[3 + k] * m1.y);
+      s[k * nI + i] = v;
+      note(k, v);
+    }
+    s[3 * nI + i] = nu;
+    note(3, nu);
+  }
+#pragma unroll
+  for (int f = 0; f < 4; ++f) {
+    for (int o = 16; o > 0; o >>= 1) big[f] = max(big[f], __shfl_xor_sync(0xffffffffu, big[f], o));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][f] = big[f];
+  }
+  __syncthreads();
+  if (threadIdx.x < 4) {
+    unsigned long long v = 0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v = max(v, red[w][threadIdx.x]);
+    unsigned long long *o = smax + 4 * level_of(L, m, id) + threadIdx.x;
+    if (v > *reinterpret_cast<volatile unsigned long long *>(o)) atomicMax(o, v);
+  }
+}
+
+// exponent e with 2^e above v (bit pattern); v = 0: any
+__device__ __forceinline__ int max_exponent(unsigned long long v) { return (int)(v >> 52) - 1022; }
+
+// fixed-point sources, node-major: fx[(cluster nI + node) 8 + 2 f + {re, im}]
+__global__ void k_src_fix(long long tot, int nI, int m, LevOff L, const double2 *__restrict__ src,
+                          const unsigned long long *__restrict__ smax, ulonglong2 *__restrict__ fx) {
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= tot) return;
+  const int f = (int)(t & 3);
+  const long long node = t >> 2;
+  const int id = (int)(node / nI), i = (int)(node - (long long)id * nI);
+  const int e = max_exponent(smax[4 * level_of(L, m, id) + f]);
+  const double2 v = src[((size_t)id * 4 + f) * nI + i];
+  fx[t] = make_ulonglong2(fix(v.x, e), fix(v.y, e));
+}
+
+// One block per (target cluster, split of its K-steps), one warp per row tile of 16 target nodes.
+// 64 source nodes at a time are staged as B fragments (digits of (Re, Im) of the 4 fields on the 8
+// columns, and of (-Im, Re) for the imaginary part of the entries); a warp streams its tile's
+// words from HBM, the next four loads in flight during the 21 products of the present ones.
+template <int MAXT, int MINB>
+__global__ void __launch_bounds__(MAXT, MINB) k_m2l_f64_digits(
+    const int *__restrict__ targets, const int *__restrict__ fptr, const int *__restrict__ fsrc,
+    const size_t *__restrict__ koff, const int *__restrict__ expo, int nI, int m, LevOff L,
+    const uint4 *__restrict__ K, const unsigned long long *__restrict__ fx,
+    const unsigned long long *__restrict__ smax, double2 *__restrict__ acc, double2 *__restrict__ more, size_t slab) {
+  __shared__ uint4 sB[kF64Nodes / 16][2][3][32];  // [step][part][digits 5 4, 3 2, 1 0][lane]
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, ntile = blockDim.x >> 5;
+  const int t = targets[blockIdx.x], k0 = fptr[t], nIe = (nI + 1) & ~1;
+  const int total = (fptr[t + 1] - k0) * nIe, nch = (total + kF64Nodes - 1) / kF64Nodes, nst = (total + 15) >> 4;
+  const int c0 = (int)((long long)nch * blockIdx.y / gridDim.y), c1 = (int)((long long)nch * (blockIdx.y + 1) / gridDim.y);
+  const uint4 *Kt = K + ((koff[t] * ntile + warp) * 8) * 32 + lane;
+  const size_t step = (size_t)ntile * 256;
+  const int st1 = min(4 * c1, nst);
+  long long hi[4] = {0, 0, 0, 0}, lo[4] = {0, 0, 0, 0};
+  uint4 nx[4];
+  if (c0 < c1)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) nx[i] = ld_stream(Kt + (size_t)(4 * c0) * step + 32 * i);
+  for (int c = c0; c < c1; ++c) {
+    __syncthreads();
+    for (int n = threadIdx.x; n < 8 * kF64Nodes; n += blockDim.x) {
+      const int node = n >> 3, col = n & 7, J = c * kF64Nodes + node;
+      unsigned long long u = kOffset;
+      if (J < total) {
+        const int k = J / nIe, i = J - k * nIe;
+        if (i < nI) u = fx[((size_t)fsrc[k0 + k] * nI + i) * 8 + col];
+      }
+      const int kk = node & 15, q = (kk & 7) >> 1, at = kk >> 3;
+      __half *r = reinterpret_cast<__half *>(&sB[node >> 4][0][0][4 * col + q]) + 2 * at + (kk & 1);
+      __half *s = reinterpret_cast<__half *>(&sB[node >> 4][1][0][4 * (col ^ 1) + q]) + 2 * at + (kk & 1);
+#pragma unroll
+      for (int d = 0; d < 6; ++d) {  // digit 5 - d: vector d / 2, words 2 (d % 2) + {0, 1}
+        const float v = (float)((int)((u >> (50 - 10 * d)) & 1023) - 512);
+        r[(d >> 1) * 256 + 4 * (d & 1)] = __float2half_rn(v);
+        s[(d >> 1) * 256 + 4 * (d & 1)] = __float2half_rn((col & 1) ? -v : v);
+      }
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int ks = 0; ks < 4; ++ks) {
+      const int st = 4 * c + ks;
+      if (st >= st1) break;
+      float D[7][4];
+#pragma unroll
+      for (int d = 0; d < 7; ++d)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) D[d][e] = 0.f;
+#pragma unroll
+      for (int part = 0; part < 2; ++part) {
+        const uint4 w[4] = {nx[0], nx[1], nx[2], nx[3]};
+        const size_t at = part == 0 ? (size_t)st * step + 128 : (size_t)min(st + 1, st1 - 1) * step;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) nx[i] = ld_stream(Kt + at + 32 * i);
+        unsigned b[12];
+#pragma unroll
+        for (int v = 0; v < 3; ++v) {
+          const uint4 x = sB[ks][part][v][lane];
+          b[4 * v] = x.x;
+          b[4 * v + 1] = x.y;
+          b[4 * v + 2] = x.z;
+          b[4 * v + 3] = x.w;
+        }
+        digit_products<5>(D, w, b);
+        digit_products<4>(D, w, b);
+        digit_products<3>(D, w, b);
+        digit_products<2>(D, w, b);
+        digit_products<1>(D, w, b);
+        digit_products<0>(D, w, b);
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        hi[e] += (long long)__float2int_rn(D[0][e]) * (1 << 20) + (long long)__float2int_rn(D[1][e]) * (1 << 10) +
+                 __float2int_rn(D[2][e]);
+        lo[e] += ((long long)__float2int_rn(D[3][e]) + __float2int_rn(D[6][e])) * (1 << 20) +
+                 (long long)__float2int_rn(D[4][e]) * (1 << 10) + __float2int_rn(D[5][e]);
+      }
+    }
+  }
+  // accumulator registers: (row g, field q) Re, Im, then (row g + 8, field q)
+  const int g = lane >> 2, f = lane & 3, row = 16 * warp + g;
+  const unsigned long long big = smax[4 * level_of(L, m, t) + f];
+  const bool bad = (big >> 52) >= 2047;  // an infinity or NaN among the sources of this level
+  const int e = expo[t] + max_exponent(big) - 2 * kFixBits + 80;
+  double v[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    v[i] = bad ? __longlong_as_double(0x7ff8000000000000ll) : scalbn((double)hi[i] + (double)lo[i] * 0x1p-30, e);
+  double2 *o = (blockIdx.y == 0 ? acc : more + (blockIdx.y - 1) * slab) + ((size_t)t * 4 + f) * nI;
+  if (row < nI) o[row] = make_double2(v[0], v[1]);
+  if (row + 8 < nI) o[row + 8] = make_double2(v[2], v[3]);
+}
+
+static LevOff lev_off(const Ctx *c) {
+  LevOff L;
+  for (int l = 0; l < 12; ++l) L.off[l] = l < (int)c->lev_off.size() ? c->lev_off[l] : c->ncl;
+  return L;
+}
+
+// K-steps before every cluster's matrices (and the total), 16 source nodes each
+static std::vector<size_t> k_steps(const Ctx *c) {
+  std::vector<int> cnt(c->ncl, 0);
+  for (int f = 0; f < c->nfar; ++f) ++cnt[c->far[3 * f + 1]];
+  std::vector<size_t> off(c->ncl + 1, 0);
+  const size_t nIe = (c->nI + 1) & ~1;
+  for (int t = 0; t < c->ncl; ++t) off[t + 1] = off[t] + (cnt[t] * nIe + 15) / 16;
+  return off;
+}
+
+size_t m2l_f64_digits_bytes(const Ctx *c) {
+  return k_steps(c).back() * (size_t)((c->nI + 15) / 16) * 4096;
+}
+
+// Evaluates and keeps the matrices in c->d_K (allocated by the caller, m2l_f64_digits_bytes).
+efie_status m2l_f64_digits_build(Ctx *c) {
+  const std::vector<size_t> off = k_steps(c);
+  EFIE_TRY(dalloc(c, &c->d_koff, off.size()));
+  EFIE_TRY(dalloc(c, &c->d_kexp, (size_t)c->ncl));
+  EFIE_TRY(dalloc(c, &c->d_smax, 4 * (size_t)(c->m + 1)));
+  EFIE_TRY(dalloc(c, &c->d_fix, (size_t)c->ncl * c->nI * 8));
+  EFIE_CUDA(cudaMemcpyAsync(c->d_koff, off.data(), sizeof(size_t) * off.size(), cudaMemcpyHostToDevice, c->stream));
+  k_K_exponent<<<c->n_m2l_targets, 128, 0, c->stream>>>(c->d_m2l_targets, c->d_far_ptr, c->d_far_src, c->nI, c->d_center,
+                                                       c->d_nodeXf, c->d_kexp); ++c->launches;
+  k_K_digits<<<c->npairs, 128, sizeof(double) * 6 * c->nI, c->stream>>>(
+      c->ncl, c->d_own_ptr, c->d_own_src, c->d_far_ptr, c->d_far_src, c->d_koff, c->d_kexp, c->nI, c->kappa, c->d_nodeX,
+      (uint4 *)c->d_K); ++c->launches;
+  EFIE_CUDA(cudaGetLastError());
+  // splits of the K-steps: enough warps for the chip when there are few targets, two staged chunks each
+  const long long warps = 16ll * c->nsm, have = (long long)c->n_m2l_targets * ((c->nI + 15) / 16);
+  const long long chunks = (long long)(off.back() / 4) / std::max(c->n_m2l_targets, 1);
+  c->f64_split = (int)std::max(1ll, std::min({2 * warps / have, chunks / 2, 16ll}));
+  if (c->f64_split > 1) {
+    const size_t n = (size_t)(c->f64_split - 1) * c->ncl * 4 * c->nI;
+    EFIE_TRY(dalloc(c, &c->d_accmore, n));
+    EFIE_CUDA(cudaMemsetAsync(c->d_accmore, 0, sizeof(double2) * n, c->stream));
+  }
+  EFIE_CUDA(cudaStreamSynchronize(c->stream));
+  return EFIE_OK;
+}
+
+// moments -> folded sources -> d_acc (and d_accmore: c->f64_split partial results)
+efie_status m2l_f64_digits_fold(Ctx *c, cudaStream_t st, const double2 *mom, double2 *src) {
+  EFIE_CUDA(cudaMemsetAsync(c->d_smax, 0, 32 * (size_t)(c->m + 1), st));
+  k_fold_max<<<c->ncl, 128, 0, st>>>(c->nI, c->m, lev_off(c), c->d_nodeD, mom, src, c->d_smax); ++c->launches;
+  const long long tot = (long long)c->ncl * c->nI * 4;
+  k_src_fix<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(tot, c->nI, c->m, lev_off(c), src, c->d_smax,
+                                                           reinterpret_cast<ulonglong2 *>(c->d_fix)); ++c->launches;
+  EFIE_CUDA(cudaGetLastError());
+  return EFIE_OK;
+}
+
+efie_status m2l_f64_digits_apply(Ctx *c, cudaStream_t st) {
+  const int ntile = (c->nI + 15) / 16;
+  const dim3 grid(c->n_m2l_targets, c->f64_split);
+  const size_t slab = (size_t)c->ncl * 4 * c->nI;
+#define EFIE_DIGITS(T, B)                                                                                        \
+  k_m2l_f64_digits<T, B><<<grid, 32 * ntile, 0, st>>>(c->d_m2l_targets, c->d_far_ptr, c->d_far_src, c->d_koff,    \
+                                                      c->d_kexp, c->nI, c->m, lev_off(c), (const uint4 *)c->d_K,  \
+                                                      c->d_fix, c->d_smax, c->d_acc, c->d_accmore, slab)
+  if (ntile <= 8) EFIE_DIGITS(256, 2);
+  else EFIE_DIGITS(640, 1);
+#undef EFIE_DIGITS
+  ++c->launches;
+  EFIE_CUDA(cudaGetLastError());
+  return EFIE_OK;
+}
+
+}  // namespace efie

@@ -218,6 +218,10 @@ efie_status dev_eval_points(Ctx *c, const std::vector<int> &patch, const std::ve
                             std::vector<double> &X, std::vector<double> *D);
 efie_status dev_cluster_geometry(Ctx *c);
 efie_status dev_near_quadrature(Ctx *c, const std::vector<NearPair> &pairs, const std::vector<int> &mirror);
+// touching pairs with factorised sums (near_touch.cu)
+bool near_touch_supported(const Ctx *c, int gdsel);
+efie_status dev_near_touch(Ctx *c, const NearPair *pairs, const int *todo, int ntodo, const int *slot, const double *x,
+                           const double *w, int gdsel);
 efie_status dev_matvec_super(Ctx *c, const double2 *xs, double2 *ys);  // ys = (N + F) xs
 efie_status dev_matvec(Ctx *c, const double2 *x, double2 *y);           // y = T^T (N+F) T x
 efie_status dev_rhs(Ctx *c, const double *dir, const double *pol, double2 *g);

@@ -17,20 +17,20 @@ namespace efie {
 // b_{f+1}^{deg-1}/(t_{f+deg+1}-t_{f+1})).  inv holds the reciprocal knot differences
 // inv[(d-1) nk + f] = 1 / (t_{f+d} - t_f) (0 where the difference is 0), nk = ncp + deg + 1,
 // so that no division is evaluated here.  Loops run to the compile-time bound GD >= deg.
-template <int GD>
-__device__ inline int dev_bspline(const double *kn, const double *inv, int deg, int ncp, double x, double *N,
-                                  double *dN) {
-  int k;
-  if (x >= kn[ncp]) {
-    k = ncp - 1;
-  } else {
-    int lo = deg, hi = ncp;  // kn[lo] <= x < kn[hi]
-    while (hi - lo > 1) {
-      int mid = (lo + hi) >> 1;
-      if (x >= kn[mid]) lo = mid; else hi = mid;
-    }
-    k = lo;
+__device__ inline int dev_span(const double *kn, int deg, int ncp, double x) {
+  if (x >= kn[ncp]) return ncp - 1;
+  int lo = deg, hi = ncp;  // kn[lo] <= x < kn[hi]
+  while (hi - lo > 1) {
+    int mid = (lo + hi) >> 1;
+    if (x >= kn[mid]) lo = mid; else hi = mid;
   }
+  return lo;
+}
+
+// the same with the span k given
+template <int GD>
+__device__ inline void dev_bspline_at(const double *kn, const double *inv, int deg, int ncp, int k, double x, double *N,
+                                      double *dN) {
   const int nk = ncp + deg + 1;
   double cur[GD + 1], prev[GD + 1];
 #pragma unroll
@@ -69,6 +69,13 @@ __device__ inline int dev_bspline(const double *kn, const double *inv, int deg, 
     }
     dN[i] = v;
   }
+}
+
+template <int GD>
+__device__ inline int dev_bspline(const double *kn, const double *inv, int deg, int ncp, double x, double *N,
+                                  double *dN) {
+  const int k = dev_span(kn, deg, ncp, x);
+  dev_bspline_at<GD>(kn, inv, deg, ncp, k, x, N, dN);
   return k;
 }
 

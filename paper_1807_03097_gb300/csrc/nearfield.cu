@@ -435,13 +435,19 @@ __global__ void k_near_mirror(int nb, const int *todo_m, const int *src_of, cons
 efie_status dev_near_quadrature(Ctx *c, const std::vector<NearPair> &pairs, const std::vector<int> &mirror) {
   if (c->nnear == 0) return EFIE_OK;
   const int nb = c->nb;
-  // pairs integrated here (the others are mirrored): touching pairs by the Duffy kernel,
-  // separated pairs by the element-table kernel when its rule fits in shared memory
-  const bool sep_fast = c->gr <= kSepMaxG;
-  std::vector<int> todo, todo_sep, todo_m, src_of;
+  // compile-time bound of the NURBS degrees of this geometry
+  int gdeg = 1;
+  for (const PatchDesc &pd : c->patches) gdeg = std::max(gdeg, std::max(pd.deg[0], pd.deg[1]));
+  const int GDsel = gdeg <= 2 ? 2 : (gdeg <= 4 ? 4 : 8);
+  // pairs integrated here (the others are mirrored): touching pairs with factorised sums (near_touch.cu)
+  // where its rule fits, separated pairs by the element-table kernel when its rule fits in shared
+  // memory, the rest by k_near_quad
+  const bool sep_fast = c->gr <= kSepMaxG, touch_fast = near_touch_supported(c, GDsel);
+  std::vector<int> todo, todo_touch, todo_sep, todo_m, src_of;
   for (int k = 0; k < c->nnear; ++k) {
     if (pairs[k].e <= pairs[k].e2) {
       if (sep_fast && pairs[k].kind == 0) todo_sep.push_back(k);
+      else if (touch_fast && pairs[k].kind != 0) todo_touch.push_back(k);
       else todo.push_back(k);
     } else {
       todo_m.push_back(k);
@@ -449,7 +455,8 @@ efie_status dev_near_quadrature(Ctx *c, const std::vector<NearPair> &pairs, cons
     }
   }
   NearPair *d_pairs = nullptr;
-  int *d_todo = nullptr, *d_todo_m = nullptr, *d_src_of = nullptr, *d_slot = nullptr, *d_sep = nullptr;
+  int *d_todo = nullptr, *d_todo_m = nullptr, *d_src_of = nullptr, *d_slot = nullptr, *d_sep = nullptr,
+      *d_touch = nullptr;
   double *d_tab = nullptr;
   std::vector<int> slot(c->nnear);
   for (int at = 0; at < c->nnear; ++at) slot[c->near_perm[at]] = at;
@@ -457,6 +464,7 @@ efie_status dev_near_quadrature(Ctx *c, const std::vector<NearPair> &pairs, cons
   EFIE_TRY(dalloc(c, &d_pairs, pairs.size()));
   EFIE_TRY(dalloc(c, &d_todo, todo.size()));
   EFIE_TRY(dalloc(c, &d_sep, todo_sep.size()));
+  EFIE_TRY(dalloc(c, &d_touch, todo_touch.size()));
   EFIE_TRY(dalloc(c, &d_todo_m, todo_m.size()));
   EFIE_TRY(dalloc(c, &d_src_of, src_of.size()));
   EFIE_TRY(dalloc(c, &d_rule, 2 * (size_t)(c->gr + c->gs)));
@@ -465,6 +473,8 @@ efie_status dev_near_quadrature(Ctx *c, const std::vector<NearPair> &pairs, cons
   EFIE_CUDA(cudaMemcpyAsync(d_slot, slot.data(), 4 * slot.size(), cudaMemcpyHostToDevice, s0));
   EFIE_CUDA(cudaMemcpyAsync(d_pairs, pairs.data(), sizeof(NearPair) * pairs.size(), cudaMemcpyHostToDevice, s0));
   if (!todo.empty()) EFIE_CUDA(cudaMemcpyAsync(d_todo, todo.data(), 4 * todo.size(), cudaMemcpyHostToDevice, s0));
+  if (!todo_touch.empty())
+    EFIE_CUDA(cudaMemcpyAsync(d_touch, todo_touch.data(), 4 * todo_touch.size(), cudaMemcpyHostToDevice, s0));
   if (!todo_sep.empty())
     EFIE_CUDA(cudaMemcpyAsync(d_sep, todo_sep.data(), 4 * todo_sep.size(), cudaMemcpyHostToDevice, s0));
   if (!todo_m.empty()) {
@@ -498,19 +508,18 @@ efie_status dev_near_quadrature(Ctx *c, const std::vector<NearPair> &pairs, cons
   A.kappa = c->kappa;
   A.h = 1.0 / c->n;
   A.blocks = c->d_nblk;
-  c->near_quad_pairs = (int)todo.size();
+  c->near_quad_pairs = (int)(todo.size() + todo_touch.size());
   c->near_sep_pairs = (int)todo_sep.size();
   c->near_quad_points = 0;
-  for (int k : todo) {
-    const int kind = pairs[k].kind, g = kind == 0 ? c->gr : c->gs;
-    const int parts = kind == 0 ? 1 : (kind == 3 ? 8 : (kind == 2 ? 6 : 4));
-    c->near_quad_points += (long long)parts * g * g * g * g;
-  }
-  // compile-time bound of the NURBS degrees of this geometry
-  int gdeg = 1;
-  for (const PatchDesc &pd : c->patches) gdeg = std::max(gdeg, std::max(pd.deg[0], pd.deg[1]));
-  const int GDsel = gdeg <= 2 ? 2 : (gdeg <= 4 ? 4 : 8);
+  for (const std::vector<int> *list : {&todo, &todo_touch})
+    for (int k : *list) {
+      const int kind = pairs[k].kind, g = kind == 0 ? c->gr : c->gs;
+      const int parts = kind == 0 ? 1 : (kind == 3 ? 8 : (kind == 2 ? 6 : 4));
+      c->near_quad_points += (long long)parts * g * g * g * g;
+    }
   EFIE_CUDA(cudaEventRecord(c->tm.ev[7], c->stream));
+  if (!todo_touch.empty())
+    EFIE_TRY(dev_near_touch(c, d_pairs, d_touch, (int)todo_touch.size(), d_slot, A.sx, A.sw, GDsel));
   bool launched = A.ntodo == 0;
 #define EFIE_QUAD(PP, GG)                                                                                 \
   if (!launched && c->p == PP && GDsel == GG) {                                                           \
@@ -588,6 +597,7 @@ efie_status dev_near_quadrature(Ctx *c, const std::vector<NearPair> &pairs, cons
   dfree(c, d_rule);
   dfree(c, d_slot);
   dfree(c, d_sep);
+  dfree(c, d_touch);
   dfree(c, d_tab);
   return EFIE_OK;
 }

@@ -131,6 +131,7 @@ struct Ctx {
   int batch_cap = 0;
   double *h_resB = nullptr;  // pinned residual estimates of a lockstep batch
   int h_resB_cap = 0;
+  int lockstep = 0;  // systems of the lockstep solve under way: its products keep one M2L kernel
   double2 *d_xB = nullptr, *d_yB = nullptr, *d_xsB = nullptr, *d_ysB = nullptr, *d_ysnB = nullptr;
   float2 *d_momB = nullptr, *d_srcB = nullptr, *d_accB = nullptr, *d_locB = nullptr;
   float2 *d_moreB = nullptr;  // [m2l_split - 1][ncl][nI][4 kMmaMaxRhs]: further splits of d_accB
@@ -170,6 +171,7 @@ struct Ctx {
   double2 *d_h2 = nullptr;    // [kr+1]
   double2 *d_part = nullptr;  // partial dot products
   double *d_gs = nullptr;     // Givens / residual state
+  double *d_nrm = nullptr;    // |w|^2 of the tiles of the orthogonalised vector
   double2 *d_w = nullptr, *d_r = nullptr, *d_b = nullptr, *d_sol = nullptr;
   double *h_res = nullptr;    // pinned host mirror of the residual estimate
   int part_cap = 0;

@@ -1485,7 +1485,9 @@ efie_status dev_matvec_batch(Ctx *c, int R, const double2 *const *X, double2 *co
   k_fold_multi<<<gtot, 256, 0, st>>>(tot, nI, R, ld, mstride, c->d_nodeD, c->d_momB, c->d_srcB); ++c->launches;
   EFIE_CUDA(cudaEventRecord(c->tm.ev[3], st));
   // a few right-hand sides, or tiles too large for tensor memory: kernel entries in mma.sync operands
-  const bool use_mma = c->opt.m2l_batch != 1 && R <= m2l_mma_rhs(c);
+  // (a lockstep solve keeps the kernel of its first product while systems drop out: the two round
+  // differently by 1e-6, which would cost GMRES iterations at a tolerance of that size)
+  const bool use_mma = c->opt.m2l_batch != 1 && std::max(R, c->lockstep) <= m2l_mma_rhs(c);
   const bool use_tc = c->opt.m2l_batch != 1 && !use_mma;
   const int nslab = use_mma && R <= kMmaMaxRhs ? c->m2l_split : 1;
   const size_t slab = (size_t)c->ncl * nI * 4 * kMmaMaxRhs;

@@ -49,9 +49,76 @@ __global__ void k_residual(int N, const double2 *__restrict__ b, double2 *__rest
 
 __global__ void k_givens_init(double *st, int kr, const double2 *h) { givens_init_dev(st, kr, h); }
 
-__global__ void k_givens_step(int j, int kr, const double2 *h1, const double2 *h2, const double2 *nrm2, double2 *H,
-                              double *st) {
-  givens_step_dev(j, kr, h1, h2, nrm2, H, st);
+// One Arnoldi step of up to S systems of one size: every operation is one launch, the system a grid
+// dimension.  w holds the product of V_j; next (if not null) receives V_{j+1} as well (the input of
+// the next product), out (if not null) the values that the host reads.
+struct GmSys {
+  double2 *V, *H, *h, *h2, *w, *part, *next;
+  double *gs, *nrm, *out;
+  int j;
+};
+template <int S>
+struct GmTab {
+  int n;
+  GmSys s[S];
+};
+
+template <int S>
+__global__ void __launch_bounds__(kDotThreads) k_gm_dot(GmTab<S> T, int N, int nchunk) {
+  const GmSys &s = T.s[blockIdx.z];
+  if ((int)blockIdx.y * kVecPerBlock <= s.j)
+    dot_partial_chunk(N, s.j + 1, blockIdx.y * kVecPerBlock, blockIdx.x, s.V, N, s.w, s.part, nchunk);
+}
+
+template <int S>
+__global__ void k_gm_final(GmTab<S> T, int nchunk, int pass) {
+  const GmSys &s = T.s[blockIdx.y];
+  const int i = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
+  if (i <= s.j) dot_final_warp(i, nchunk, s.part, pass == 0 ? s.h : s.h2);
+}
+
+template <int S>
+__global__ void __launch_bounds__(kCombThreads) k_gm_combine(GmTab<S> T, int N, int pass) {
+  const GmSys &s = T.s[blockIdx.y];
+  combine_tile(N, blockIdx.x * kCombRows, s.j + 1, s.V, N, pass == 0 ? s.h : s.h2, -1.0, s.w, pass == 0 ? nullptr : s.nrm);
+}
+
+template <int S>
+__global__ void __launch_bounds__(kGivThreads) k_gm_givens(GmTab<S> T, int kr, int ntile) {
+  const GmSys &s = T.s[blockIdx.x];
+  givens_step_block(s.j, kr, s.h, s.h2, s.nrm, ntile, s.H, s.gs);
+  if (threadIdx.x == 0 && s.out) {
+    s.out[0] = s.gs[0];
+    s.out[1] = s.gs[1];
+  }
+}
+
+template <int S>
+__global__ void k_gm_scale(GmTab<S> T, int N) {
+  const GmSys &s = T.s[blockIdx.y];
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= N) return;
+  const double2 v = scaled_entry(s.w[t], s.gs[0]);
+  s.V[(size_t)(s.j + 1) * N + t] = v;
+  if (s.next) s.next[t] = v;
+}
+
+// CGS2, Givens and the next Krylov vector of the systems of T (jmax: their largest j)
+template <int S>
+static efie_status arnoldi_step(Ctx *c, const GmTab<S> &T, int N, int kr, int jmax) {
+  cudaStream_t st = c->stream;
+  const unsigned n = T.n, nchunk = (N + kChunk - 1) / kChunk, ntile = (N + kCombRows - 1) / kCombRows;
+  const unsigned groups = (jmax + kVecPerBlock) / kVecPerBlock;  // of jmax + 1 vectors
+  for (int pass = 0; pass < 2; ++pass) {
+    k_gm_dot<S><<<dim3(nchunk, groups, n), kDotThreads, 0, st>>>(T, N, nchunk);
+    k_gm_final<S><<<dim3(groups, n), 256, 0, st>>>(T, nchunk, pass);
+    k_gm_combine<S><<<dim3(ntile, n), kCombThreads, 0, st>>>(T, N, pass);
+  }
+  k_gm_givens<S><<<n, kGivThreads, 0, st>>>(T, kr, ntile);
+  k_gm_scale<S><<<dim3((N + 255) / 256, n), 256, 0, st>>>(T, N);
+  c->launches += 8;
+  EFIE_CUDA(cudaGetLastError());
+  return EFIE_OK;
 }
 
 __global__ void k_backsolve(int jd, int kr, const double2 *H, const double *st, double2 *y) {
@@ -85,35 +152,40 @@ void drop_product_graph(Ctx *c) {
   dfree(c, c->d_mvin);
 }
 
-// out = A in for the single-system solver as one CUDA-graph launch: the product chain (about
+// The product of the single-system solver as one CUDA-graph launch: the product chain (about
 // 20 small kernels around the M2L, near field on the second stream) is captured once per setup
 // with input d_mvin and output d_w, and replayed, without the launch gaps between its kernels.
+static efie_status gmres_product_prepare(Ctx *c) {
+  if (c->g_mv) return EFIE_OK;
+  cudaStream_t st = c->stream;
+  EFIE_TRY(dalloc(c, &c->d_mvin, (size_t)c->ndof));
+  EFIE_CUDA(cudaMemsetAsync(c->d_mvin, 0, sizeof(double2) * (size_t)c->ndof, st));
+  EFIE_TRY(dev_matvec(c, c->d_mvin, c->d_w));  // buffers created on first use exist before the capture
+  EFIE_CUDA(cudaStreamSynchronize(st));
+  const long long l0 = c->launches;
+  EFIE_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+  const efie_status s = dev_matvec(c, c->d_mvin, c->d_w);
+  cudaGraph_t g = nullptr;
+  const cudaError_t e = cudaStreamEndCapture(st, &g);
+  c->mv_kernels = c->launches - l0;
+  c->launches = l0;
+  if (s != EFIE_OK) {
+    if (g) cudaGraphDestroy(g);
+    return s;
+  }
+  EFIE_CUDA(e);
+  const cudaError_t ei = cudaGraphInstantiate(&c->g_mv, g, 0);
+  cudaGraphDestroy(g);
+  if (ei != cudaSuccess) c->g_mv = nullptr;
+  EFIE_CUDA(ei);
+  return EFIE_OK;
+}
+
+// out = A in; in = null: the input is in d_mvin already (gmres_product_prepare has run)
 static efie_status gmres_product(Ctx *c, const double2 *in, double2 *out) {
   cudaStream_t st = c->stream;
   const size_t bytes = sizeof(double2) * (size_t)c->ndof;
-  if (!c->g_mv) {
-    EFIE_TRY(dalloc(c, &c->d_mvin, (size_t)c->ndof));
-    EFIE_CUDA(cudaMemsetAsync(c->d_mvin, 0, bytes, st));
-    EFIE_TRY(dev_matvec(c, c->d_mvin, c->d_w));  // buffers created on first use exist before the capture
-    EFIE_CUDA(cudaStreamSynchronize(st));
-    const long long l0 = c->launches;
-    EFIE_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-    const efie_status s = dev_matvec(c, c->d_mvin, c->d_w);
-    cudaGraph_t g = nullptr;
-    const cudaError_t e = cudaStreamEndCapture(st, &g);
-    c->mv_kernels = c->launches - l0;
-    c->launches = l0;
-    if (s != EFIE_OK) {
-      if (g) cudaGraphDestroy(g);
-      return s;
-    }
-    EFIE_CUDA(e);
-    const cudaError_t ei = cudaGraphInstantiate(&c->g_mv, g, 0);
-    cudaGraphDestroy(g);
-    if (ei != cudaSuccess) c->g_mv = nullptr;
-    EFIE_CUDA(ei);
-  }
-  EFIE_CUDA(cudaMemcpyAsync(c->d_mvin, in, bytes, cudaMemcpyDeviceToDevice, st));
+  if (in) EFIE_CUDA(cudaMemcpyAsync(c->d_mvin, in, bytes, cudaMemcpyDeviceToDevice, st));
   EFIE_CUDA(cudaGraphLaunch(c->g_mv, st));
   if (out != c->d_w) EFIE_CUDA(cudaMemcpyAsync(out, c->d_w, bytes, cudaMemcpyDeviceToDevice, st));
   c->launches += c->mv_kernels;
@@ -136,6 +208,7 @@ efie_status dev_gmres(Ctx *c, const double2 *b, double2 *x, int *its_out, double
     EFIE_TRY(dalloc(c, &c->d_w, N));
     EFIE_TRY(dalloc(c, &c->d_r, N));
     EFIE_TRY(dalloc(c, &c->d_sol, (size_t)kr + 1));
+    EFIE_TRY(dalloc(c, &c->d_nrm, (size_t)(N + kCombRows - 1) / kCombRows));
   }
   if (!c->h_res) c->h_res = static_cast<double *>(pinned_get(4 * sizeof(double)));
   if (!c->h_res) {
@@ -154,6 +227,8 @@ efie_status dev_gmres(Ctx *c, const double2 *b, double2 *x, int *its_out, double
   int its = 0, conv = 0;
   double res = bn;
   if (bn == 0.0) conv = 1;
+  if (!conv) EFIE_TRY(gmres_product_prepare(c));
+  EFIE_TRY(ensure_part(c, N, kr + 1));
   bool first = true;
   while (!conv && its < c->opt.gmres_maxit) {
     // r = b - A x
@@ -167,6 +242,7 @@ efie_status dev_gmres(Ctx *c, const double2 *b, double2 *x, int *its_out, double
     EFIE_TRY(dots(c, N, 1, c->d_r, N, c->d_r, c->d_h));
     k_givens_init<<<1, 1, 0, st>>>(c->d_gs, kr, c->d_h); ++c->launches;
     k_scale_copy<<<grid, blk, 0, st>>>(N, c->d_r, c->d_gs, 0, V); ++c->launches;
+    EFIE_CUDA(cudaMemcpyAsync(c->d_mvin, V, sizeof(double2) * N, cudaMemcpyDeviceToDevice, st));
     EFIE_CUDA(cudaMemcpyAsync(c->h_res, c->d_gs, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
     EFIE_CUDA(cudaStreamSynchronize(st));
     res = c->h_res[1];
@@ -176,18 +252,10 @@ efie_status dev_gmres(Ctx *c, const double2 *b, double2 *x, int *its_out, double
     }
     int jd = 0;
     for (int j = 0; j < kr && its < c->opt.gmres_maxit; ++j) {
-      double2 *vj = V + (size_t)j * N;
-      EFIE_TRY(gmres_product(c, vj, c->d_w));
+      EFIE_TRY(gmres_product(c, nullptr, c->d_w));
       ++its;
-      // CGS2
-      EFIE_TRY(dots(c, N, j + 1, V, N, c->d_w, c->d_h));
-      k_combine<<<(N + kCombRows - 1) / kCombRows, kCombThreads, 0, st>>>(N, j + 1, V, N, c->d_h, -1.0, c->d_w); ++c->launches;
-      EFIE_TRY(dots(c, N, j + 1, V, N, c->d_w, c->d_h2));
-      k_combine<<<(N + kCombRows - 1) / kCombRows, kCombThreads, 0, st>>>(N, j + 1, V, N, c->d_h2, -1.0, c->d_w); ++c->launches;
-      EFIE_TRY(dots(c, N, 1, c->d_w, N, c->d_w, c->d_h2 + kr));
-      k_givens_step<<<1, 1, 0, st>>>(j, kr, c->d_h, c->d_h2, c->d_h2 + kr, c->d_H, c->d_gs); ++c->launches;
-      k_scale_copy<<<grid, blk, 0, st>>>(N, c->d_w, c->d_gs, 0, V + (size_t)(j + 1) * N); ++c->launches;
-      EFIE_CUDA(cudaGetLastError());
+      const GmTab<1> T = {1, {{V, c->d_H, c->d_h, c->d_h2, c->d_w, c->d_part, c->d_mvin, c->d_gs, c->d_nrm, nullptr, j}}};
+      EFIE_TRY(arnoldi_step<1>(c, T, N, kr, j));
       EFIE_CUDA(cudaMemcpyAsync(c->h_res, c->d_gs, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
       EFIE_CUDA(cudaStreamSynchronize(st));
       res = c->h_res[1];
@@ -237,13 +305,15 @@ efie_status dev_norms(Ctx *c, int N, const double2 *v, double *out) {
 namespace efie {
 
 namespace {
+constexpr int kArnBatch = 64;  // systems of one Arnoldi launch (kernel arguments: 5 KB)
 enum Phase { kStart, kArnoldi, kConfirm, kDone };
 
 struct GSys {
   const double2 *b = nullptr;
   double2 *x = nullptr;
   double2 *V = nullptr, *H = nullptr, *h = nullptr, *h2 = nullptr, *w = nullptr, *r = nullptr, *sol = nullptr;
-  double *gs = nullptr;
+  double2 *part = nullptr;
+  double *gs = nullptr, *nrm = nullptr;
   double bn = 0, target = 0, res = 0;
   int its = 0, conv = 0, j = 0, phase = kStart;
   bool r_ready = false;  // r holds b (first cycle) or b - A x (after a failed check)
@@ -253,7 +323,8 @@ struct GSys {
 
 size_t gmres_batch_bytes_per_system(const Ctx *c) {
   const size_t N = c->ndof, kr = std::max(1, std::min(c->opt.gmres_restart, c->opt.gmres_maxit));
-  return 16 * ((kr + 1) * N + (kr + 1) * kr + 3 * (kr + 1) + 2 * N) + 8 * (5 * kr + 4);
+  const size_t nchunk = (N + kChunk - 1) / kChunk, ntile = (N + kCombRows - 1) / kCombRows;
+  return 16 * ((kr + 1) * N + (kr + 1) * kr + 3 * (kr + 1) + 2 * N + nchunk * (kr + 1 + kVecPerBlock)) + 8 * (5 * kr + 4 + ntile + 4);
 }
 
 efie_status dev_gmres_batch(Ctx *c, int R, const double2 *const *b, double2 *const *x, int *its_out,
@@ -264,6 +335,11 @@ efie_status dev_gmres_batch(Ctx *c, int R, const double2 *const *b, double2 *con
   cudaStream_t st = c->stream;
   const int blk = 256, grid = (N + blk - 1) / blk;
   DevTemp mem;
+  struct Hint {
+    Ctx *c;
+    ~Hint() { c->lockstep = 0; }
+  } hint{c};
+  c->lockstep = R;
   std::vector<GSys> S(R);
   for (int i = 0; i < R; ++i) {
     GSys &s = S[i];
@@ -277,7 +353,11 @@ efie_status dev_gmres_batch(Ctx *c, int R, const double2 *const *b, double2 *con
     EFIE_TRY(mem.get(c, &s.w, (size_t)N));
     EFIE_TRY(mem.get(c, &s.r, (size_t)N));
     EFIE_TRY(mem.get(c, &s.gs, (size_t)2 + 5 * kr + 2));
+    EFIE_TRY(mem.get(c, &s.part, (size_t)((N + kChunk - 1) / kChunk) * (kr + 1 + kVecPerBlock)));
+    EFIE_TRY(mem.get(c, &s.nrm, (size_t)(N + kCombRows - 1) / kCombRows));
   }
+  double *d_out = nullptr;  // [R][4]: values read by the host after an Arnoldi step
+  EFIE_TRY(mem.get(c, &d_out, 4 * (size_t)R));
   if (c->h_resB_cap < 4 * R) {
     pinned_put(c->h_resB);
     c->h_resB_cap = 0;
@@ -336,22 +416,26 @@ efie_status dev_gmres_batch(Ctx *c, int R, const double2 *const *b, double2 *con
       if (S[i].phase != kArnoldi) {
         k_residual<<<grid, blk, 0, st>>>(N, S[i].b, S[i].r); ++c->launches;
       }
+    // the systems in an Arnoldi step together, up to kArnBatch at a time
+    for (int i = 0; i < R;) {
+      GmTab<kArnBatch> T;
+      T.n = 0;
+      int jmax = 0;
+      for (; i < R && T.n < kArnBatch; ++i) {
+        const GSys &s = S[i];
+        if (s.phase != kArnoldi) continue;
+        T.s[T.n++] = {s.V, s.H, s.h, s.h2, s.w, s.part, nullptr, s.gs, s.nrm, d_out + 4 * i, s.j};
+        jmax = std::max(jmax, s.j);
+      }
+      if (T.n > 0) EFIE_TRY(arnoldi_step<kArnBatch>(c, T, N, kr, jmax));
+    }
+    EFIE_CUDA(cudaMemcpyAsync(hr, d_out, 4 * R * sizeof(double), cudaMemcpyDeviceToHost, st));
     for (int i = 0; i < R; ++i) {
       GSys &s = S[i];
       if (s.phase == kStart) {
         EFIE_TRY(dots(c, N, 1, s.r, N, s.r, s.h));
         k_givens_init<<<1, 1, 0, st>>>(s.gs, kr, s.h); ++c->launches;
         k_scale_copy<<<grid, blk, 0, st>>>(N, s.r, s.gs, 0, s.V); ++c->launches;
-        EFIE_CUDA(cudaMemcpyAsync(hr + 4 * i, s.gs, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
-      } else if (s.phase == kArnoldi) {
-        const int j = s.j;
-        EFIE_TRY(dots(c, N, j + 1, s.V, N, s.w, s.h));
-        k_combine<<<(N + kCombRows - 1) / kCombRows, kCombThreads, 0, st>>>(N, j + 1, s.V, N, s.h, -1.0, s.w); ++c->launches;
-        EFIE_TRY(dots(c, N, j + 1, s.V, N, s.w, s.h2));
-        k_combine<<<(N + kCombRows - 1) / kCombRows, kCombThreads, 0, st>>>(N, j + 1, s.V, N, s.h2, -1.0, s.w); ++c->launches;
-        EFIE_TRY(dots(c, N, 1, s.w, N, s.w, s.h2 + kr));
-        k_givens_step<<<1, 1, 0, st>>>(j, kr, s.h, s.h2, s.h2 + kr, s.H, s.gs); ++c->launches;
-        k_scale_copy<<<grid, blk, 0, st>>>(N, s.w, s.gs, 0, s.V + (size_t)(j + 1) * N); ++c->launches;
         EFIE_CUDA(cudaMemcpyAsync(hr + 4 * i, s.gs, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
       } else if (s.phase == kConfirm) {
         EFIE_TRY(dots(c, N, 1, s.r, N, s.r, s.h));

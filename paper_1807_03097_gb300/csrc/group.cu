@@ -11,7 +11,7 @@
 //   post:     residuals, CGS2 (two passes), norms, Givens rotations, the next Krylov vector and
 //             the residual estimates of all systems, then one device-to-host copy of them.
 // The per-system work of pre and post runs in one launch per operation over a table of chunks
-// of 2048 vector entries (system, chunk), with the same arithmetic in the same order as the
+// of 512 vector entries (system, chunk), with the same arithmetic in the same order as the
 // single-context solver (gmres_ops.cuh), so that a system solved in a group follows the same
 // iterates as alone up to the rounding of its products.
 #include <algorithm>
@@ -43,7 +43,7 @@ enum : int {
 struct GSysD {
   int N, kr, mode, j, jd, nchunk;
   double2 *V, *H, *h, *h2, *sol, *w, *r, *x, *b, *px, *py, *part;
-  double *gs;
+  double *gs, *nrm;
 };
 
 __global__ void k_g_backsolve(const GSysD *__restrict__ T) {
@@ -85,8 +85,7 @@ __global__ void __launch_bounds__(kDotThreads) k_g_unpack(const GSysD *__restric
   }
 }
 
-// vectors of the dot products of pass 0 (first CGS pass, or a norm), 1 (second CGS pass),
-// 2 (norm of the orthogonalised vector)
+// vectors of the dot products of pass 0 (first CGS pass, or a norm), 1 (second CGS pass)
 __device__ __forceinline__ int dot_operands(const GSysD &s, int pass, const double2 *&V, const double2 *&w,
                                             double2 *&dst) {
   V = w = nullptr;
@@ -111,15 +110,10 @@ __device__ __forceinline__ int dot_operands(const GSysD &s, int pass, const doub
     return 0;
   }
   if (!(s.mode & G_ARN)) return 0;
-  if (pass == 1) {
-    V = s.V;
-    w = s.w;
-    dst = s.h2;
-    return s.j + 1;
-  }
-  V = w = s.w;
-  dst = s.h2 + s.kr;
-  return 1;
+  V = s.V;
+  w = s.w;
+  dst = s.h2;
+  return s.j + 1;
 }
 
 __global__ void __launch_bounds__(kDotThreads) k_g_dot_partial(const GSysD *__restrict__ T, const int *__restrict__ csys,
@@ -147,16 +141,17 @@ __global__ void __launch_bounds__(kCombThreads) k_g_combine(const GSysD *__restr
   if (!(s.mode & G_ARN)) return;
   const int t0 = cidx[blockIdx.x] * kChunk + blockIdx.y * kCombRows;
   if (t0 >= s.N) return;
-  combine_tile(s.N, t0, s.j + 1, s.V, (size_t)s.N, pass == 0 ? s.h : s.h2, -1.0, s.w);
+  combine_tile(s.N, t0, s.j + 1, s.V, (size_t)s.N, pass == 0 ? s.h : s.h2, -1.0, s.w,
+               pass == 0 ? nullptr : s.nrm);
 }
 
-// one thread per system: Givens step or start, then the values the host reads
-__global__ void k_g_givens(const GSysD *__restrict__ T, int nsys, double *__restrict__ out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nsys) return;
-  const GSysD &s = T[i];
-  if (s.mode & G_ARN) givens_step_dev(s.j, s.kr, s.h, s.h2, s.h2 + s.kr, s.H, s.gs);
-  else if (s.mode & G_START) givens_init_dev(s.gs, s.kr, s.h);
+// one block per system: Givens step or start, then the values the host reads
+__global__ void __launch_bounds__(kGivThreads) k_g_givens(const GSysD *__restrict__ T, double *__restrict__ out) {
+  const int i = blockIdx.x;
+  const GSysD s = T[i];
+  if (s.mode & G_ARN) givens_step_block(s.j, s.kr, s.h, s.h2, s.nrm, (s.N + kCombRows - 1) / kCombRows, s.H, s.gs);
+  else if (s.mode & G_START && threadIdx.x == 0) givens_init_dev(s.gs, s.kr, s.h);
+  if (threadIdx.x > 0) return;
   if (s.mode & (G_ARN | G_START)) {
     out[2 * i] = s.gs[0];
     out[2 * i + 1] = s.gs[1];
@@ -219,7 +214,7 @@ struct Group {
 
 namespace {
 
-constexpr int kPreKernels = 2, kPostKernels = 11;
+constexpr int kPreKernels = 2, kPostKernels = 9;
 
 efie_status capture_graph(Group *g, cudaGraphExec_t *out, efie_status (*body)(Group *)) {
   Ctx *c = &g->gc;
@@ -257,14 +252,13 @@ efie_status body_post(Group *g) {
   Ctx *c = &g->gc;
   cudaStream_t st = c->stream;
   k_g_unpack<<<g->nchunks, kDotThreads, 0, st>>>(g->d_tab, g->d_csys, g->d_cidx);
-  for (int pass = 0; pass < 3; ++pass) {
-    const int groups = pass == 2 ? 1 : std::min(32, (g->kr_max + 1 + kVecPerBlock - 1) / kVecPerBlock);
+  for (int pass = 0; pass < 2; ++pass) {
+    const int groups = std::min(32, (g->kr_max + 1 + kVecPerBlock - 1) / kVecPerBlock);
     k_g_dot_partial<<<dim3(g->nchunks, groups), kDotThreads, 0, st>>>(g->d_tab, g->d_csys, g->d_cidx, pass);
     k_g_dot_final<<<g->nsys, 256, 0, st>>>(g->d_tab, pass);
-    if (pass < 2)
-      k_g_combine<<<dim3(g->nchunks, kChunk / kCombRows), kCombThreads, 0, st>>>(g->d_tab, g->d_csys, g->d_cidx, pass);
+    k_g_combine<<<dim3(g->nchunks, kChunk / kCombRows), kCombThreads, 0, st>>>(g->d_tab, g->d_csys, g->d_cidx, pass);
   }
-  k_g_givens<<<(g->nsys + 127) / 128, 128, 0, st>>>(g->d_tab, g->nsys, g->d_out);
+  k_g_givens<<<g->nsys, kGivThreads, 0, st>>>(g->d_tab, g->d_out);
   k_g_scale<<<g->nchunks, kDotThreads, 0, st>>>(g->d_tab, g->d_csys, g->d_cidx);
   EFIE_CUDA(cudaMemcpyAsync(g->h_out, g->d_out, sizeof(double) * 2 * g->nsys, cudaMemcpyDeviceToHost, st));
   EFIE_CUDA(cudaGetLastError());
@@ -482,6 +476,7 @@ efie_status efie_group_solve(efie_group *grp, const double *const *b, double *co
     EFIE_TRY(mem.get(c, &d.r, N));
     EFIE_TRY(mem.get(c, &d.gs, 2 + 5 * kr + 2));
     EFIE_TRY(mem.get(c, &d.part, (size_t)d.nchunk * (kr + 1 + kVecPerBlock)));
+    EFIE_TRY(mem.get(c, &d.nrm, (size_t)(s.N + kCombRows - 1) / kCombRows));
     if (ptr_kind == EFIE_PTR_DEVICE) {
       d.b = reinterpret_cast<double2 *>(const_cast<double *>(b[i]));
       d.x = reinterpret_cast<double2 *>(x[i]);

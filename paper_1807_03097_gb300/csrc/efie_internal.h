@@ -138,8 +138,8 @@ struct Ctx {
   int *d_tc_err = nullptr;   // set by a tensor-core M2L whose pipeline wait ran out
   int *d_near_ptr = nullptr, *d_near_src = nullptr;  // CSR by target element
   double2 *d_nblk = nullptr;  // [nnear][nb (col)][nb (row)]
-  float2 *d_nblkf = nullptr;  // FP32 copy of the blocks (mixed-precision apply)
-  float2 *d_xsf = nullptr;    // x* in FP32 for the FP32 block product [nsup]
+  float2 *d_nblkf = nullptr;  // FP32 copy of the blocks (mixed-precision apply; 8 x 8 blocks: in row pairs)
+  float2 *d_xsf = nullptr;    // x* in FP32 for the FP32 block product [nsup] (8 x 8 blocks: hi + lo, [nsup][2] float4)
   std::vector<int> near_perm;  // CSR position -> index in nearl
 
   // tables on the device

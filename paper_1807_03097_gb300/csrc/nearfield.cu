@@ -781,6 +781,102 @@ __global__ void __launch_bounds__(128) k_near_apply_w(int nE, int per, const int
   }
 }
 
+// (h, l) += b x with the product's and the sum's rounding errors and b xlo kept in l (Dekker's
+// product by FMA, Knuth's two-sum), two rows at once
+__device__ __forceinline__ void acc_exact(float2 &h, float2 &l, float2 b, float2 x, float2 xlo) {
+  const float2 m1 = make_float2(-1.f, -1.f), z = make_float2(-0.f, -0.f);
+  const float2 t = __ffma2_rn(b, x, z);
+  const float2 e = __ffma2_rn(b, x, __fmul2_rn(t, m1));
+  const float2 s = __fadd2_rn(h, t);
+  const float2 bp = __ffma2_rn(h, m1, s);
+  const float2 u = __fadd2_rn(h, __ffma2_rn(s, m1, bp));  // h - (s - bp)
+  const float2 v = __ffma2_rn(bp, m1, t);
+  l = __fadd2_rn(__ffma2_rn(b, xlo, l), __fadd2_rn(__fadd2_rn(u, v), e));
+  h = s;
+}
+
+// (h, l) += (h2, l2)
+__device__ __forceinline__ void acc_pair(float2 &h, float2 &l, float2 h2, float2 l2) {
+  const float2 m1 = make_float2(-1.f, -1.f);
+  const float2 s = __fadd2_rn(h, h2);
+  const float2 bp = __ffma2_rn(h, m1, s);
+  const float2 u = __fadd2_rn(h, __ffma2_rn(s, m1, bp));
+  const float2 v = __ffma2_rn(bp, m1, h2);
+  l = __fadd2_rn(__fadd2_rn(l, l2), __fadd2_rn(u, v));
+  h = s;
+}
+
+__device__ __forceinline__ float2 shfl2(float2 v, int src) {
+  return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
+}
+
+// x* as hi + lo in FP32, each number twice for the packed products: y[2 i] = (Re, Re, Im, Im) of hi,
+// y[2 i + 1] of lo.
+__global__ void k_vec_to_f32x2(int n, const double2 *__restrict__ x, float4 *__restrict__ y) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const float re = (float)x[i].x, im = (float)x[i].y;
+  const float rl = (float)(x[i].x - (double)re), il = (float)(x[i].y - (double)im);
+  y[2 * i] = make_float4(re, re, im, im);
+  y[2 * i + 1] = make_float4(rl, rl, il, il);
+}
+
+// The same for 8 x 8 blocks (p = 1) with every rounding error kept: sums are carried as hi + lo, 24 packed
+// FP32 instructions an entry.  The rounding of x* to FP32 and of the products was the largest noise of the
+// mixed product: at low frequency, where the 1/kappa^2 part cancels, it stopped GMRES at 1e-6 (cube,
+// kappa = 0.8, 768 unknowns, 12 incidences: 114 to 2 060 iterations, 524 on average; now 90 or 91).
+// The 8 x 8 blocks have the room for it (53 us before and after at 6 144 elements: HBM and
+// latency bound); with 18 x 18 blocks the packed FP32 pipe would bound the kernel (63 -> 241 us).
+// Blocks are stored per column in row pairs, float4 (Re 2k, Re 2k+1, Im 2k, Im 2k+1); lane l owns rows
+// 2 (l % 4), 2 (l % 4) + 1 and column l / 4, so one load a lane takes a block, BIF of them in flight.
+template <int BIF>
+__global__ void __launch_bounds__(128) k_near_apply_8(int nE, int per, const int *__restrict__ ptr,
+                                                      const int *__restrict__ src, const float4 *__restrict__ blocks,
+                                                      const float4 *__restrict__ xs, double2 *__restrict__ ysn) {
+  const int lane = threadIdx.x & 31;
+  const int rp = lane & 3, col = lane >> 2;
+  const int wid = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int e0 = wid * per, e1 = min(e0 + per, nE);
+  const float2 zero = make_float2(0.f, 0.f);
+  for (int e = e0; e < e1; ++e) {
+    float2 hr = zero, lr = zero, hi = zero, li = zero;  // rows 2 rp, 2 rp + 1: Re, Im
+    const int k0 = ptr[e], k1 = ptr[e + 1];
+    for (int k = k0; k < k1; k += BIF) {
+      float4 b[BIF], xh[BIF], xl[BIF];
+#pragma unroll
+      for (int i = 0; i < BIF; ++i) {
+        const int kk = min(k + i, k1 - 1);
+        const float4 *x = xs + ((size_t)src[kk] * 8 + col) * 2;
+        b[i] = k + i < k1 ? __ldcs(blocks + (size_t)kk * 32 + col * 4 + rp) : make_float4(0.f, 0.f, 0.f, 0.f);
+        xh[i] = x[0];
+        xl[i] = x[1];
+      }
+#pragma unroll
+      for (int i = 0; i < BIF; ++i) {
+        const float2 xr = make_float2(xh[i].x, xh[i].y), xi = make_float2(xh[i].z, xh[i].w);
+        const float2 br = make_float2(b[i].x, b[i].y), bi = make_float2(b[i].z, b[i].w);
+        const float2 nb = make_float2(-bi.x, -bi.y);
+        acc_exact(hr, lr, br, xr, make_float2(xl[i].x, xl[i].y));
+        acc_exact(hi, li, br, xi, make_float2(xl[i].z, xl[i].w));
+        acc_exact(hr, lr, nb, xi, make_float2(xl[i].z, xl[i].w));
+        acc_exact(hi, li, bi, xr, make_float2(xl[i].x, xl[i].y));
+      }
+    }
+    // the 8 columns in a fixed order
+    const float2 hr0 = hr, lr0 = lr, hi0 = hi, li0 = li;
+#pragma unroll
+    for (int g = 1; g < 8; ++g) {
+      const int from = (rp + 4 * g) & 31;
+      acc_pair(hr, lr, shfl2(hr0, from), shfl2(lr0, from));
+      acc_pair(hi, li, shfl2(hi0, from), shfl2(li0, from));
+    }
+    if (lane < 4) {
+      ysn[(size_t)e * 8 + 2 * lane] = make_double2((double)hr.x + (double)lr.x, (double)hi.x + (double)li.x);
+      ysn[(size_t)e * 8 + 2 * lane + 1] = make_double2((double)hr.y + (double)lr.y, (double)hi.y + (double)li.y);
+    }
+  }
+}
+
 // The same product for several right-hand sides (FP32 blocks, mixed form): each block is read
 // once for a group of up to RB right-hand sides (grid dimension y), which divides the HBM
 // traffic of the near field by RB.  Vectors of right-hand side r start at r * vstride.
@@ -838,7 +934,12 @@ __global__ void __launch_bounds__(32 * kApplyWarps) k_near_apply_multi(int nE, i
 #pragma unroll
         for (int t = 0; t < RPL; ++t) {
           const int rr = rl + GS * t;
-          b[t] = (act && rr < NB) ? B[cc * NB + rr] : make_float2(0.f, 0.f);
+          if (NB == 8) {  // row pairs: Re, Re, Im, Im
+            const float *v = reinterpret_cast<const float *>(B + cc * NB + (rr & ~1)) + (rr & 1);
+            b[t] = act ? make_float2(v[0], v[2]) : make_float2(0.f, 0.f);
+          } else {
+            b[t] = (act && rr < NB) ? B[cc * NB + rr] : make_float2(0.f, 0.f);
+          }
         }
 #pragma unroll
         for (int j = 0; j < RB; ++j) {
@@ -892,10 +993,23 @@ __global__ void k_blocks_to_f32(size_t n, const double2 *__restrict__ in, float2
   if (i < n) out[i] = make_float2((float)in[i].x, (float)in[i].y);
 }
 
+// in row pairs (8 x 8 blocks)
+__global__ void k_blocks_to_f32_pairs(size_t n, const double2 *__restrict__ in, float4 *__restrict__ out) {
+  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const double2 a = in[2 * i], b = in[2 * i + 1];
+  out[i] = make_float4((float)a.x, (float)b.x, (float)a.y, (float)b.y);
+}
+
 efie_status dev_near_blocks_f32(Ctx *c) {
   size_t n = (size_t)c->nnear * c->nb * c->nb;
   EFIE_TRY(dalloc(c, &c->d_nblkf, n));
-  k_blocks_to_f32<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(n, c->d_nblk, c->d_nblkf); ++c->launches;
+  if (c->nb == 8)
+    k_blocks_to_f32_pairs<<<(unsigned)((n / 2 + 255) / 256), 256, 0, c->stream>>>(
+        n / 2, c->d_nblk, reinterpret_cast<float4 *>(c->d_nblkf));
+  else
+    k_blocks_to_f32<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(n, c->d_nblk, c->d_nblkf);
+  ++c->launches;
   EFIE_CUDA(cudaGetLastError());
   return EFIE_OK;
 }
@@ -935,19 +1049,23 @@ efie_status dev_near_apply(Ctx *c, const double2 *xs, double2 *ysn, cudaStream_t
   const bool f32 = c->opt.precision == EFIE_MIXED_FP32 && c->d_nblkf;
   const int threads = 32 * kApplyWarps;
   if (f32) {
-    const unsigned grid = (unsigned)c->nE;
     const float4 *B = reinterpret_cast<const float4 *>(c->d_nblkf);
-    bool done = c->nb == 8 || c->nb == 18 || c->nb == 32;
+    const bool done = c->nb == 8 || c->nb == 18 || c->nb == 32;
     if (done) {
-      if (!c->d_xsf) EFIE_TRY(dalloc(c, &c->d_xsf, (size_t)c->nsup));
-      k_vec_to_f32<<<(c->nsup + 255) / 256, 256, 0, st>>>(c->nsup, xs, c->d_xsf);
+      // 8 x 8 blocks: two float4 per entry, else one float2
+      if (!c->d_xsf) EFIE_TRY(dalloc(c, &c->d_xsf, (c->nb == 8 ? 4 : 1) * (size_t)c->nsup));
+      const unsigned gv = (unsigned)((c->nsup + 255) / 256);
+      if (c->nb == 8) k_vec_to_f32x2<<<gv, 256, 0, st>>>(c->nsup, xs, reinterpret_cast<float4 *>(c->d_xsf));
+      else k_vec_to_f32<<<gv, 256, 0, st>>>(c->nsup, xs, c->d_xsf);
       ++c->launches;
       const float2 *xf = c->d_xsf;
       // one warp per element, the same number of elements per warp: about 20 warps per SM
       const int per = (c->nE + c->nsm * 20 - 1) / (c->nsm * 20);
       const int nw = (c->nE + per - 1) / per;
       const unsigned gw = (unsigned)((nw + 3) / 4);
-      if (c->nb == 8) k_near_apply_w<8, 2><<<gw, 128, 0, st>>>(c->nE, per, c->d_near_ptr, c->d_near_src, B, xf, ysn);
+      if (c->nb == 8)
+        k_near_apply_8<4><<<gw, 128, 0, st>>>(c->nE, per, c->d_near_ptr, c->d_near_src, B,
+                                              reinterpret_cast<const float4 *>(xf), ysn);
       else if (c->nb == 18) k_near_apply_w<18, 2><<<gw, 128, 0, st>>>(c->nE, per, c->d_near_ptr, c->d_near_src, B, xf, ysn);
       else k_near_apply_w<32, 2><<<gw, 128, 0, st>>>(c->nE, per, c->d_near_ptr, c->d_near_src, B, xf, ysn);
       ++c->launches;

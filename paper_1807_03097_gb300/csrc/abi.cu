@@ -31,7 +31,7 @@ void release_device(Ctx *c) {
   dfree(c, c->d_nodeX); dfree(c, c->d_nodeD); dfree(c, c->d_nodeXf); dfree(c, c->d_center);
   dfree(c, c->d_far_ptr); dfree(c, c->d_far_src); dfree(c, c->d_m2l_targets);
   dfree(c, c->d_near_ptr); dfree(c, c->d_near_src); dfree(c, c->d_nblk); dfree(c, c->d_nblkf); dfree(c, c->d_xsf);
-  dfree(c, c->d_M); dfree(c, c->d_Md); dfree(c, c->d_E); dfree(c, c->d_Mf); dfree(c, c->d_Mdf); dfree(c, c->d_Ef);
+  dfree(c, c->d_M); dfree(c, c->d_Md); dfree(c, c->d_E); dfree(c, c->d_Mf); dfree(c, c->d_Mdf); dfree(c, c->d_Ef); dfree(c, c->d_nodeDf);
   dfree(c, c->d_x); dfree(c, c->d_y); dfree(c, c->d_xs); dfree(c, c->d_ys); dfree(c, c->d_ysn);
   dfree(c, c->d_mom); dfree(c, c->d_src); dfree(c, c->d_acc); dfree(c, c->d_loc);
   dfree(c, c->d_momf); dfree(c, c->d_srcf); dfree(c, c->d_locf); dfree(c, c->d_accm); dfree(c, c->d_accf);

@@ -144,7 +144,7 @@ struct Ctx {
 
   // tables on the device
   double *d_M = nullptr, *d_Md = nullptr, *d_E = nullptr;
-  float *d_Mf = nullptr, *d_Mdf = nullptr, *d_Ef = nullptr;
+  float *d_Mf = nullptr, *d_Mdf = nullptr, *d_Ef = nullptr, *d_nodeDf = nullptr;  // FP32 copies (mixed form)
   Tables tab;
 
   // work vectors (FP64)
@@ -250,10 +250,17 @@ struct MmaArgs {
 int m2l_mma_splits(const Ctx *c);
 int m2l_mma_rhs(const Ctx *c);  // right-hand sides up to which a batch takes it
 efie_status launch_m2l_mma(Ctx *c, cudaStream_t st, const MmaArgs &A);
+// product stages around the M2L (tree.cu): xs -> sources, M2L results -> ys; `nrhs` vectors nsup apart
+efie_status tree_up_f32(Ctx *c, cudaStream_t st, int nrhs, const double2 *xs, float2 *mom, float2 *src, int ld);
+efie_status tree_up_f64(Ctx *c, cudaStream_t st, const double2 *xs, double2 *mom, double2 *src, unsigned long long *smax);
+efie_status tree_down_f32(Ctx *c, cudaStream_t st, int nrhs, float2 *acc, int ld, const float2 *more, int ldm, int nslab,
+                          size_t slab, float2 *loc, double2 *ys);
+efie_status tree_down_f64(Ctx *c, cudaStream_t st, double2 *acc, const double2 *more, int nslab, size_t slab, double2 *loc,
+                          double2 *ys);
 // FP64 M2L from kept matrices in digits on the FP16 tensor cores (m2l_f64.cu)
 size_t m2l_f64_digits_bytes(const Ctx *c);
 efie_status m2l_f64_digits_build(Ctx *c);
-efie_status m2l_f64_digits_fold(Ctx *c, cudaStream_t st, const double2 *mom, double2 *src);
+efie_status m2l_f64_digits_fix(Ctx *c, cudaStream_t st, const double2 *src);
 efie_status m2l_f64_digits_apply(Ctx *c, cudaStream_t st);
 // tensor-core M2L of a batch (m2l_tc.cu)
 bool m2l_tc_supported(const Ctx *c);

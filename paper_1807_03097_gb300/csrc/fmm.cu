@@ -22,43 +22,70 @@ namespace efie {
 
 efie_status dev_near_apply(Ctx *c, const double2 *xs, double2 *ysn, cudaStream_t st);
 
-template <class R> struct Cx;
-template <> struct Cx<double> { using T = double2; };
-template <> struct Cx<float> { using T = float2; };
-template <class R> using C2 = typename Cx<R>::T;
-template <class R> __device__ inline C2<R> mk(R a, R b) { C2<R> v; v.x = a; v.y = b; return v; }
-
 // ------------------------------------------------------------------------ T and T^T
+// One launch for up to kTMax vectors (grid dimension y).
+constexpr int kTMax = 64;
+struct TVecs {
+  const double2 *in[kTMax];
+  double2 *out[kTMax];
+};
+
 __global__ void k_gather(int nrow, const int *__restrict__ ptr, const int *__restrict__ col,
-                         const double *__restrict__ val, const double2 *__restrict__ x, double2 *__restrict__ xs) {
+                         const double *__restrict__ val, TVecs V) {
   int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= nrow) return;
+  const double2 *__restrict__ x = V.in[blockIdx.y];
   double2 s = make_double2(0.0, 0.0);
   for (int k = ptr[r]; k < ptr[r + 1]; ++k) {
     double2 v = x[col[k]];
     s.x += val[k] * v.x;
     s.y += val[k] * v.y;
   }
-  xs[r] = s;
+  V.out[blockIdx.y][r] = s;
 }
 
+// y = T^T (ys + ysn), ysn a second part (or null), vstride apart for the vectors of a batch.  Eight
+// lanes a row: a row has up to ~100 entries (p = 3), and a few thousand rows with a thread each
+// left most SMs idle (33 us a vector at 3 200 unknowns).
 __global__ void k_scatter(int ndof, const int *__restrict__ ptr, const int *__restrict__ row,
                           const double *__restrict__ val, const double2 *__restrict__ ys,
-                          const double2 *__restrict__ ysn, double2 *__restrict__ y) {
-  int d = blockIdx.x * blockDim.x + threadIdx.x;
-  if (d >= ndof) return;
+                          const double2 *__restrict__ ysn, size_t vstride, TVecs V) {
+  const int d = (blockIdx.x * blockDim.x + threadIdx.x) >> 3, lane = threadIdx.x & 7;
   double2 s = make_double2(0.0, 0.0);
-  for (int k = ptr[d]; k < ptr[d + 1]; ++k) {
-    double2 v = ys[row[k]];
-    if (ysn) {
-      double2 w = ysn[row[k]];
-      v.x += w.x;
-      v.y += w.y;
+  if (d < ndof) {
+    const size_t o = blockIdx.y * vstride;
+    for (int k = ptr[d] + lane; k < ptr[d + 1]; k += 8) {
+      double2 v = ys[o + row[k]];
+      if (ysn) {
+        double2 w = ysn[o + row[k]];
+        v.x += w.x;
+        v.y += w.y;
+      }
+      s.x += val[k] * v.x;
+      s.y += val[k] * v.y;
     }
-    s.x += val[k] * v.x;
-    s.y += val[k] * v.y;
   }
-  y[d] = s;
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) {
+    s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+    s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+  }
+  if (d < ndof && lane == 0) V.out[blockIdx.y][d] = s;
+}
+
+static efie_status launch_gather(Ctx *c, cudaStream_t st, int R, const TVecs &V) {
+  k_gather<<<dim3((c->nsup + 255) / 256, R), 256, 0, st>>>(c->nsup, c->d_tg_ptr, c->d_tg_col, c->d_tg_val, V);
+  ++c->launches;
+  EFIE_CUDA(cudaGetLastError());
+  return EFIE_OK;
+}
+
+static efie_status launch_scatter(Ctx *c, cudaStream_t st, int R, const double2 *ys, const double2 *ysn, size_t vstride,
+                                  const TVecs &V) {
+  k_scatter<<<dim3((c->ndof + 31) / 32, R), 256, 0, st>>>(c->ndof, c->d_ts_ptr, c->d_ts_col, c->d_ts_val, ys, ysn, vstride, V);
+  ++c->launches;
+  EFIE_CUDA(cudaGetLastError());
+  return EFIE_OK;
 }
 
 __global__ void k_add(int n, double2 *a, const double2 *b) {
@@ -67,162 +94,6 @@ __global__ void k_add(int n, double2 *a, const double2 *b) {
     a[i].x += b[i].x;
     a[i].y += b[i].y;
   }
-}
-
-// ------------------------------------------------------------------------ a4 leaf moments
-// mu_beta(m) = h^2 sum_ab M[m1][a] M[m2][b] x*_{beta,b,a}
-// nu(m)      = h sum_ab (Md[m1][a] M[m2][b] x*_{0,b,a} + M[m1][a] Md[m2][b] x*_{1,b,a})
-template <class R>
-__global__ void k_leaf_moments(int nE, int leaf_off, int p1, int q1, R h, const double *__restrict__ Mt,
-                               const double *__restrict__ Mdt, const double2 *__restrict__ xs, C2<R> *__restrict__ mom,
-                               size_t xstride = 0, size_t mstride = 0) {
-  int e = blockIdx.x;
-  if (e >= nE) return;
-  xs += blockIdx.y * xstride;  // right-hand side blockIdx.y of a batch
-  mom += blockIdx.y * mstride;
-  int nI = q1 * q1;
-  __shared__ R sM[kMaxQ1 * kMaxP1], sMd[kMaxQ1 * kMaxP1];
-  __shared__ C2<R> sx[2 * kMaxP1 * kMaxP1];
-  __shared__ C2<R> T0[kMaxP1 * kMaxQ1], T1[kMaxP1 * kMaxQ1], Td[kMaxP1 * kMaxQ1];
-  for (int i = threadIdx.x; i < q1 * p1; i += blockDim.x) {
-    sM[i] = (R)Mt[i];
-    sMd[i] = (R)Mdt[i];
-  }
-  for (int i = threadIdx.x; i < 2 * p1 * p1; i += blockDim.x) {
-    double2 v = xs[(size_t)e * 2 * p1 * p1 + i];
-    sx[i] = mk<R>((R)v.x, (R)v.y);
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < p1 * q1; i += blockDim.x) {
-    int b = i / q1, m1 = i % q1;
-    C2<R> a0 = mk<R>(0, 0), a1 = mk<R>(0, 0), ad = mk<R>(0, 0);
-    for (int a = 0; a < p1; ++a) {
-      R M = sM[m1 * p1 + a], Md = sMd[m1 * p1 + a];
-      C2<R> x0 = sx[b * p1 + a], x1 = sx[p1 * p1 + b * p1 + a];
-      a0.x += M * x0.x; a0.y += M * x0.y;
-      a1.x += M * x1.x; a1.y += M * x1.y;
-      ad.x += Md * x0.x; ad.y += Md * x0.y;
-    }
-    T0[i] = a0;
-    T1[i] = a1;
-    Td[i] = ad;
-  }
-  __syncthreads();
-  C2<R> *out = mom + (size_t)(leaf_off + e) * 3 * nI;
-  R h2 = h * h;
-  for (int mi = threadIdx.x; mi < nI; mi += blockDim.x) {
-    int m1 = mi % q1, m2 = mi / q1;
-    C2<R> u0 = mk<R>(0, 0), u1 = mk<R>(0, 0), v = mk<R>(0, 0);
-    for (int b = 0; b < p1; ++b) {
-      R M = sM[m2 * p1 + b], Md = sMd[m2 * p1 + b];
-      C2<R> t0 = T0[b * q1 + m1], t1 = T1[b * q1 + m1], td = Td[b * q1 + m1];
-      u0.x += M * t0.x; u0.y += M * t0.y;
-      u1.x += M * t1.x; u1.y += M * t1.y;
-      v.x += M * td.x + Md * t1.x; v.y += M * td.y + Md * t1.y;
-    }
-    out[mi] = mk<R>(h2 * u0.x, h2 * u0.y);
-    out[nI + mi] = mk<R>(h2 * u1.x, h2 * u1.y);
-    out[2 * nI + mi] = mk<R>(h * v.x, h * v.y);
-  }
-}
-
-// ------------------------------------------------------------------------ a5 M2M
-// parent(f, m2, m1) = sum_c sum_{m2'} E[c2][m2][m2'] sum_{m1'} E[c1][m1][m1'] child_c(f, m2', m1')
-template <class R>
-__global__ void k_m2m(int nparent, int par_off, int ch_off, int q1, const double *__restrict__ Et,
-                      C2<R> *__restrict__ mom, size_t mstride = 0) {
-  int pid = blockIdx.x;
-  if (pid >= nparent) return;
-  mom += blockIdx.y * mstride;
-  int nI = q1 * q1;
-  extern __shared__ unsigned char smraw[];
-  R *sE = (R *)smraw;                                      // [2][q1][q1]
-  C2<R> *ch = (C2<R> *)(smraw + sizeof(double) * 2 * kMaxQ1 * kMaxQ1);  // [4][3][nI]
-  C2<R> *T = ch + 12 * nI;                                 // [4][3][q1 (m2')][q1 (m1)]
-  for (int i = threadIdx.x; i < 2 * q1 * q1; i += blockDim.x) sE[i] = (R)Et[i];
-  // children of parent (patch j, K) at level l are 4K + c at level l + 1: contiguous
-  const C2<R> *cm = mom + (size_t)(ch_off + 4 * pid) * 3 * nI;
-  for (int i = threadIdx.x; i < 12 * nI; i += blockDim.x) ch[i] = cm[i];
-  __syncthreads();
-  for (int i = threadIdx.x; i < 12 * nI; i += blockDim.x) {
-    int cf = i / nI, rem = i % nI, m2p = rem / q1, m1 = rem % q1;
-    int cidx = cf / 3, c1 = cidx & 1;
-    C2<R> s = mk<R>(0, 0);
-    const C2<R> *src = ch + cf * nI + m2p * q1;
-    for (int m1p = 0; m1p < q1; ++m1p) {
-      R e = sE[(c1 * q1 + m1) * q1 + m1p];
-      s.x += e * src[m1p].x;
-      s.y += e * src[m1p].y;
-    }
-    T[i] = s;
-  }
-  __syncthreads();
-  C2<R> *out = mom + (size_t)(par_off + pid) * 3 * nI;
-  for (int i = threadIdx.x; i < 3 * nI; i += blockDim.x) {
-    int f = i / nI, rem = i % nI, m2 = rem / q1, m1 = rem % q1;
-    C2<R> s = mk<R>(0, 0);
-    for (int cidx = 0; cidx < 4; ++cidx) {
-      int c2 = cidx >> 1;
-      const C2<R> *tt = T + (cidx * 3 + f) * nI;
-      for (int m2p = 0; m2p < q1; ++m2p) {
-        R e = sE[(c2 * q1 + m2) * q1 + m2p];
-        s.x += e * tt[m2p * q1 + m1].x;
-        s.y += e * tt[m2p * q1 + m1].y;
-      }
-    }
-    out[i] = s;
-  }
-}
-
-// ------------------------------------------------------------------------ fold / unfold
-template <class R>
-__global__ void k_fold(long long tot, int nI, const double *__restrict__ nodeD, const C2<R> *__restrict__ mom,
-                       C2<R> *__restrict__ src) {
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= tot) return;
-  int id = (int)(t / nI), mi = (int)(t % nI);
-  const double *D = nodeD + 6 * t;
-  const C2<R> *mm = mom + (size_t)id * 3 * nI;
-  C2<R> m0 = mm[mi], m1 = mm[nI + mi];
-  C2<R> *s = src + (size_t)id * 4 * nI;
-  for (int k = 0; k < 3; ++k) {
-    R d1 = (R)D[k], d2 = (R)D[3 + k];
-    s[k * nI + mi] = mk<R>(d1 * m0.x + d2 * m1.x, d1 * m0.y + d2 * m1.y);
-  }
-  s[3 * nI + mi] = mm[2 * nI + mi];
-}
-
-// acc plus nslab - 1 further partial results of the M2L in `more` (splits of the source lists)
-template <class R, class A>
-__global__ void k_unfold(long long tot, int nI, R ik2, const double *__restrict__ nodeD, const A *__restrict__ acc,
-                         const A *__restrict__ more, int nslab, size_t slab, C2<R> *__restrict__ loc) {
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= tot) return;
-  int id = (int)(t / nI), mi = (int)(t % nI);
-  const double *D = nodeD + 6 * t;
-  A sum[4];
-  for (int k = 0; k < 4; ++k) {
-    const size_t at = ((size_t)id * 4 + k) * nI + mi;
-    sum[k] = acc[at];
-    for (int j = 1; j < nslab; ++j) {
-      const A b = more[(j - 1) * slab + at];
-      sum[k].x += b.x;
-      sum[k].y += b.y;
-    }
-  }
-  R l0x = 0, l0y = 0, l1x = 0, l1y = 0;
-  for (int k = 0; k < 3; ++k) {
-    A v = sum[k];
-    l0x += (R)D[k] * (R)v.x;
-    l0y += (R)D[k] * (R)v.y;
-    l1x += (R)D[3 + k] * (R)v.x;
-    l1y += (R)D[3 + k] * (R)v.y;
-  }
-  C2<R> *l = loc + (size_t)id * 3 * nI;
-  l[mi] = mk<R>(l0x, l0y);
-  l[nI + mi] = mk<R>(l1x, l1y);
-  A dv = sum[3];
-  l[2 * nI + mi] = mk<R>(-ik2 * (R)dv.x, -ik2 * (R)dv.y);
 }
 
 // ------------------------------------------------------------------------ a6 M2L (FP64)
@@ -276,25 +147,8 @@ __global__ void k_m2l_f64(const int *__restrict__ targets, const int *__restrict
 }
 
 // ------------------------------------------------------------------------ a6 M2L (FP32, node-major)
-// Folded source fields of the FP32 path, node-major: src[(id nI + m) 2] = (u_x, u_y),
+// Folded source fields and results of the FP32 path, node-major: src[(id nI + m) 2] = (u_x, u_y),
 // src[(id nI + m) 2 + 1] = (u_z, nu).
-__global__ void k_fold_f32n(long long tot, int nI, const double *__restrict__ nodeD, const float2 *__restrict__ mom,
-                            float4 *__restrict__ src) {
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= tot) return;
-  int id = (int)(t / nI), mi = (int)(t % nI);
-  const double *D = nodeD + 6 * t;
-  const float2 *mm = mom + (size_t)id * 3 * nI;
-  float2 m0 = mm[mi], m1 = mm[nI + mi], nu = mm[2 * nI + mi];
-  float u[6];
-  for (int k = 0; k < 3; ++k) {
-    float d1 = (float)D[k], d2 = (float)D[3 + k];
-    u[2 * k] = d1 * m0.x + d2 * m1.x;
-    u[2 * k + 1] = d1 * m0.y + d2 * m1.y;
-  }
-  src[2 * t] = make_float4(u[0], u[1], u[2], u[3]);
-  src[2 * t + 1] = make_float4(u[4], u[5], nu.x, nu.y);
-}
 
 // Per far pair (CSR order): d = c_t - c_s and r0 = |d| in FP32, e^{i kappa r0} / (4 pi) from
 // FP64.  Computed once at setup.
@@ -540,34 +394,6 @@ __global__ void k_m2l_sym_reduce(int nred, const int *__restrict__ red, const in
   acc[2 * ((size_t)c * nI + m) + 1] = make_float4(h[4] + l[4], h[5] + l[5], h[6] + l[6], h[7] + l[7]);
 }
 
-// acc: `nslab` partial results of the M2L (splits of the source lists), `slab` float4 apart,
-// added in order
-__global__ void k_unfold_f32n(long long tot, int nI, float ik2, const double *__restrict__ nodeD,
-                              const float4 *__restrict__ acc, int nslab, size_t slab, float2 *__restrict__ loc) {
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= tot) return;
-  int id = (int)(t / nI), mi = (int)(t % nI);
-  const double *D = nodeD + 6 * t;
-  float4 u = acc[2 * t], v = acc[2 * t + 1];
-  for (int k = 1; k < nslab; ++k) {
-    const float4 a = acc[k * slab + 2 * t], b = acc[k * slab + 2 * t + 1];
-    u = make_float4(u.x + a.x, u.y + a.y, u.z + a.z, u.w + a.w);
-    v = make_float4(v.x + b.x, v.y + b.y, v.z + b.z, v.w + b.w);
-  }
-  float cr[3] = {u.x, u.z, v.x}, ci[3] = {u.y, u.w, v.y};
-  float l0x = 0, l0y = 0, l1x = 0, l1y = 0;
-  for (int k = 0; k < 3; ++k) {
-    l0x += (float)D[k] * cr[k];
-    l0y += (float)D[k] * ci[k];
-    l1x += (float)D[3 + k] * cr[k];
-    l1y += (float)D[3 + k] * ci[k];
-  }
-  float2 *l = loc + (size_t)id * 3 * nI;
-  l[mi] = make_float2(l0x, l0y);
-  l[nI + mi] = make_float2(l1x, l1y);
-  l[2 * nI + mi] = make_float2(-ik2 * v.z, -ik2 * v.w);
-}
-
 // ------------------------------------------------------------------------ a6 M2L, stored matrices
 // When they fit in device memory, the coupling matrices of all admissible blocks are
 // evaluated once at setup, K[k][m'][m] = G(F_t(x_m) - F_s(x_m')) / (4 pi) (column m'
@@ -729,110 +555,6 @@ __global__ void __launch_bounds__(128) k_m2l_f64_stored(const int *__restrict__ 
     if (lane < T && mi < nI)
 #pragma unroll
       for (int q = 0; q < 4; ++q) acc[(size_t)t * 4 * nI + q * nI + mi] = make_double2(ar[j][q], ai[j][q]);
-  }
-}
-
-// ------------------------------------------------------------------------ a7 L2L
-// child_c(f, m2', m1') += sum_{m2} E[c2][m2][m2'] sum_{m1} E[c1][m1][m1'] parent(f, m2, m1)
-template <class R>
-__global__ void k_l2l(int nparent, int par_off, int ch_off, int q1, const double *__restrict__ Et,
-                      C2<R> *__restrict__ loc, size_t mstride = 0) {
-  int pid = blockIdx.x;
-  if (pid >= nparent) return;
-  loc += blockIdx.y * mstride;
-  int nI = q1 * q1;
-  extern __shared__ unsigned char smraw[];
-  R *sE = (R *)smraw;
-  C2<R> *par = (C2<R> *)(smraw + sizeof(double) * 2 * kMaxQ1 * kMaxQ1);  // [3][nI]
-  C2<R> *T = par + 3 * nI;                                              // [2][3][q1 m2][q1 m1']
-  for (int i = threadIdx.x; i < 2 * q1 * q1; i += blockDim.x) sE[i] = (R)Et[i];
-  const C2<R> *pl = loc + (size_t)(par_off + pid) * 3 * nI;
-  for (int i = threadIdx.x; i < 3 * nI; i += blockDim.x) par[i] = pl[i];
-  __syncthreads();
-  for (int i = threadIdx.x; i < 6 * nI; i += blockDim.x) {
-    int c1 = i / (3 * nI), rem = i % (3 * nI), f = rem / nI, r2 = rem % nI, m2 = r2 / q1, m1p = r2 % q1;
-    C2<R> s = mk<R>(0, 0);
-    const C2<R> *pp = par + f * nI + m2 * q1;
-    for (int m1 = 0; m1 < q1; ++m1) {
-      R e = sE[(c1 * q1 + m1) * q1 + m1p];
-      s.x += e * pp[m1].x;
-      s.y += e * pp[m1].y;
-    }
-    T[i] = s;
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < 12 * nI; i += blockDim.x) {
-    int cidx = i / (3 * nI), rem = i % (3 * nI), f = rem / nI, r2 = rem % nI, m2p = r2 / q1, m1p = r2 % q1;
-    int c1 = cidx & 1, c2 = cidx >> 1;
-    const C2<R> *tt = T + (c1 * 3 + f) * nI;
-    C2<R> s = mk<R>(0, 0);
-    for (int m2 = 0; m2 < q1; ++m2) {
-      R e = sE[(c2 * q1 + m2) * q1 + m2p];
-      s.x += e * tt[m2 * q1 + m1p].x;
-      s.y += e * tt[m2 * q1 + m1p].y;
-    }
-    C2<R> *cl = loc + (size_t)(ch_off + 4 * pid + cidx) * 3 * nI;
-    C2<R> o = cl[f * nI + r2];
-    o.x += s.x;
-    o.y += s.y;
-    cl[f * nI + r2] = o;
-  }
-}
-
-// ------------------------------------------------------------------------ a8 leaf evaluation
-// y*_{0,b,a} = h^2 sum_m M[m1][a] M[m2][b] l_0(m) + h sum_m Md[m1][a] M[m2][b] l_div(m)
-// y*_{1,b,a} = h^2 sum_m M[m1][a] M[m2][b] l_1(m) + h sum_m M[m1][a] Md[m2][b] l_div(m)
-template <class R>
-__global__ void k_leaf_eval(int nE, int leaf_off, int p1, int q1, R h, const double *__restrict__ Mt,
-                            const double *__restrict__ Mdt, const C2<R> *__restrict__ loc, double2 *__restrict__ ys,
-                            size_t mstride = 0, size_t ystride = 0) {
-  int e = blockIdx.x;
-  if (e >= nE) return;
-  loc += blockIdx.y * mstride;  // right-hand side blockIdx.y of a batch
-  ys += blockIdx.y * ystride;
-  int nI = q1 * q1;
-  __shared__ R sM[kMaxQ1 * kMaxP1], sMd[kMaxQ1 * kMaxP1];
-  __shared__ C2<R> R0[kMaxQ1 * kMaxP1], R1[kMaxQ1 * kMaxP1], R2[kMaxQ1 * kMaxP1], Rd[kMaxQ1 * kMaxP1];
-  for (int i = threadIdx.x; i < q1 * p1; i += blockDim.x) {
-    sM[i] = (R)Mt[i];
-    sMd[i] = (R)Mdt[i];
-  }
-  __syncthreads();
-  const C2<R> *l = loc + (size_t)(leaf_off + e) * 3 * nI;
-  for (int i = threadIdx.x; i < q1 * p1; i += blockDim.x) {
-    int m2 = i / p1, a = i % p1;
-    C2<R> s0 = mk<R>(0, 0), s1 = s0, s2 = s0, sd = s0;
-    for (int m1 = 0; m1 < q1; ++m1) {
-      R M = sM[m1 * p1 + a], Md = sMd[m1 * p1 + a];
-      C2<R> v0 = l[m2 * q1 + m1], v1 = l[nI + m2 * q1 + m1], v2 = l[2 * nI + m2 * q1 + m1];
-      s0.x += M * v0.x; s0.y += M * v0.y;
-      s1.x += M * v1.x; s1.y += M * v1.y;
-      s2.x += M * v2.x; s2.y += M * v2.y;
-      sd.x += Md * v2.x; sd.y += Md * v2.y;
-    }
-    R0[i] = s0;
-    R1[i] = s1;
-    R2[i] = s2;
-    Rd[i] = sd;
-  }
-  __syncthreads();
-  R h2 = h * h;
-  for (int i = threadIdx.x; i < 2 * p1 * p1; i += blockDim.x) {
-    int al = i / (p1 * p1), b = (i / p1) % p1, a = i % p1;
-    R ax = 0, ay = 0;
-    for (int m2 = 0; m2 < q1; ++m2) {
-      R M = sM[m2 * p1 + b], Md = sMd[m2 * p1 + b];
-      if (al == 0) {
-        C2<R> u = R0[m2 * p1 + a], d = Rd[m2 * p1 + a];
-        ax += h2 * M * u.x + h * M * d.x;
-        ay += h2 * M * u.y + h * M * d.y;
-      } else {
-        C2<R> u = R1[m2 * p1 + a], d = R2[m2 * p1 + a];
-        ax += h2 * M * u.x + h * Md * d.x;
-        ay += h2 * M * u.y + h * Md * d.y;
-      }
-    }
-    ys[(size_t)e * 2 * p1 * p1 + i] = make_double2((double)ax, (double)ay);
   }
 }
 
@@ -1088,73 +810,42 @@ static efie_status m2l_f32_tables(Ctx *c) {
   if (c->opt.m2l_pairs == 2 && c->d_back) EFIE_TRY(m2l_autotune(c));
   return EFIE_OK;
 }
-static size_t m2m_smem(int q1, size_t csz) { return sizeof(double) * 2 * kMaxQ1 * kMaxQ1 + csz * 24 * q1 * q1; }
-static size_t l2l_smem(int q1, size_t csz) { return sizeof(double) * 2 * kMaxQ1 * kMaxQ1 + csz * 9 * q1 * q1; }
 
-template <class R>
-static efie_status far_chain(Ctx *c, const double2 *xs, double2 *ys, C2<R> *mom, C2<R> *srcv, C2<R> *loc,
-                             const double *M, const double *Md, const double *E) {
-  const int nI = c->nI, q1 = c->q1, p1 = c->p1, m = c->m;
-  const R h = (R)(1.0 / c->n);
+static efie_status far_chain_f32(Ctx *c, const double2 *xs, double2 *ys) {
   cudaStream_t st = c->stream;
-  size_t csz = sizeof(C2<R>);
-  k_leaf_moments<R><<<c->nE, 128, 0, st>>>(c->nE, c->lev_off[m], p1, q1, h, M, Md, xs, mom); ++c->launches;
-  for (int l = m - 1; l >= 0; --l) {
-    int npar = c->np << (2 * l);
-    k_m2m<R><<<npar, 128, m2m_smem(q1, csz), st>>>(npar, c->lev_off[l], c->lev_off[l + 1], q1, E, mom); ++c->launches;
-  }
-  long long tot = (long long)c->ncl * nI;
-  const unsigned gtot = (unsigned)((tot + 255) / 256);
-  if (sizeof(R) == 8 && c->k_digits) {
-    EFIE_TRY(m2l_f64_digits_fold(c, st, (const double2 *)mom, (double2 *)srcv));
-  } else if (sizeof(R) == 8) {
-    k_fold<double><<<gtot, 256, 0, st>>>(tot, nI, c->d_nodeD, (const double2 *)mom, (double2 *)srcv); ++c->launches;
-  } else {
-    k_fold_f32n<<<gtot, 256, 0, st>>>(tot, nI, c->d_nodeD, (const float2 *)mom, c->d_srcf); ++c->launches;
-  }
+  float2 *src = reinterpret_cast<float2 *>(c->d_srcf), *acc = reinterpret_cast<float2 *>(c->d_accf);
+  const size_t slab = (size_t)c->ncl * 4 * c->nI;
+  EFIE_TRY(tree_up_f32(c, st, 1, xs, c->d_momf, src, 4));
+  cudaEventRecord(c->tm.ev[3], st);
+  int nslab = 1;
+  if (c->n_m2l_targets > 0 && c->k_stored) EFIE_TRY(launch_m2l_stored(c, st, true));
+  else if (c->n_m2l_targets > 0) EFIE_TRY(launch_m2l_f32(c, st, &nslab));
+  cudaEventRecord(c->tm.ev[4], st);
+  return tree_down_f32(c, st, 1, acc, 4, acc + slab, 4, nslab, slab, c->d_locf, ys);
+}
+
+static efie_status far_chain_f64(Ctx *c, const double2 *xs, double2 *ys) {
+  cudaStream_t st = c->stream;
+  const int nI = c->nI;
+  if (c->k_digits) EFIE_CUDA(cudaMemsetAsync(c->d_smax, 0, 32 * (size_t)(c->m + 1), st));
+  EFIE_TRY(tree_up_f64(c, st, xs, c->d_mom, c->d_src, c->k_digits ? c->d_smax : nullptr));
+  if (c->k_digits) EFIE_TRY(m2l_f64_digits_fix(c, st, c->d_src));
   cudaEventRecord(c->tm.ev[3], st);
   int nslab = 1;
   if (c->n_m2l_targets > 0 && c->k_digits) {
     EFIE_TRY(m2l_f64_digits_apply(c, st));
     nslab = c->f64_split;
   } else if (c->n_m2l_targets > 0 && c->k_stored) {
-    EFIE_TRY(launch_m2l_stored(c, st, sizeof(R) == 4));
+    EFIE_TRY(launch_m2l_stored(c, st, false));
   } else if (c->n_m2l_targets > 0) {
-    if (sizeof(R) == 8) {
-      int thr = ((nI + 31) / 32) * 32;
-      size_t sm = sizeof(double) * (3 * nI + 1) + sizeof(double2) * 4 * nI;
-      k_m2l_f64<<<c->n_m2l_targets, thr, sm, st>>>(c->d_m2l_targets, c->d_far_ptr, c->d_far_src, nI, c->kappa,
-                                                   c->d_nodeX, (const double2 *)srcv, c->d_acc); ++c->launches;
-    } else {
-      EFIE_TRY(launch_m2l_f32(c, st, &nslab));
-    }
+    int thr = ((nI + 31) / 32) * 32;
+    size_t sm = sizeof(double) * (3 * nI + 1) + sizeof(double2) * 4 * nI;
+    k_m2l_f64<<<c->n_m2l_targets, thr, sm, st>>>(c->d_m2l_targets, c->d_far_ptr, c->d_far_src, nI, c->kappa,
+                                                 c->d_nodeX, c->d_src, c->d_acc); ++c->launches;
+    EFIE_CUDA(cudaGetLastError());
   }
   cudaEventRecord(c->tm.ev[4], st);
-  if (sizeof(R) == 8) {
-    k_unfold<double, double2><<<gtot, 256, 0, st>>>(tot, nI, 1.0 / (c->kappa * c->kappa), c->d_nodeD, c->d_acc,
-                                                    c->d_accmore, nslab, (size_t)c->ncl * 4 * nI, (double2 *)loc);
-    ++c->launches;
-  } else {
-    k_unfold_f32n<<<gtot, 256, 0, st>>>(tot, nI, (float)(1.0 / (c->kappa * c->kappa)), c->d_nodeD, c->d_accf,
-                                        nslab, (size_t)c->ncl * 2 * nI, (float2 *)loc); ++c->launches;
-  }
-  for (int l = 0; l < m; ++l) {
-    int npar = c->np << (2 * l);
-    k_l2l<R><<<npar, 128, l2l_smem(q1, csz), st>>>(npar, c->lev_off[l], c->lev_off[l + 1], q1, E, loc); ++c->launches;
-  }
-  k_leaf_eval<R><<<c->nE, 128, 0, st>>>(c->nE, c->lev_off[m], p1, q1, h, M, Md, loc, ys); ++c->launches;
-  EFIE_CUDA(cudaGetLastError());
-  return EFIE_OK;
-}
-
-efie_status dev_set_kernel_attrs(Ctx *c) {
-  size_t mx = 0;
-  for (size_t csz : {sizeof(double2), sizeof(float2)}) mx = std::max(mx, m2m_smem(c->q1, csz));
-  EFIE_CUDA(cudaFuncSetAttribute(k_m2m<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx));
-  EFIE_CUDA(cudaFuncSetAttribute(k_m2m<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx));
-  EFIE_CUDA(cudaFuncSetAttribute(k_l2l<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx));
-  EFIE_CUDA(cudaFuncSetAttribute(k_l2l<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mx));
-  return EFIE_OK;
+  return tree_down_f64(c, st, c->d_acc, c->d_accmore, nslab, (size_t)c->ncl * 4 * nI, c->d_loc, ys);
 }
 
 // ys = (N + F) xs; the near field runs on the second stream, concurrently with the far
@@ -1167,9 +858,9 @@ static efie_status superspace_apply(Ctx *c, const double2 *xs, double2 *ys, doub
   EFIE_CUDA(cudaEventRecord(c->tm.ev[2], c->stream2));
   EFIE_CUDA(cudaEventRecord(c->join, c->stream2));
   if (c->opt.precision == EFIE_MIXED_FP32) {
-    EFIE_TRY(far_chain<float>(c, xs, ys, c->d_momf, nullptr, c->d_locf, c->d_M, c->d_Md, c->d_E));
+    EFIE_TRY(far_chain_f32(c, xs, ys));
   } else {
-    EFIE_TRY(far_chain<double>(c, xs, ys, c->d_mom, c->d_src, c->d_loc, c->d_M, c->d_Md, c->d_E));
+    EFIE_TRY(far_chain_f64(c, xs, ys));
   }
   EFIE_CUDA(cudaEventRecord(c->tm.ev[5], st));
   EFIE_CUDA(cudaStreamWaitEvent(st, c->join, 0));
@@ -1186,31 +877,33 @@ efie_status dev_matvec_super(Ctx *c, const double2 *xs, double2 *ys) {
   return EFIE_OK;
 }
 
+static TVecs one_vec(const double2 *in, double2 *out) {
+  TVecs V;
+  V.in[0] = in;
+  V.out[0] = out;
+  return V;
+}
+
 efie_status dev_matvec(Ctx *c, const double2 *x, double2 *y) {
   cudaStream_t st = c->stream;
   EFIE_CUDA(cudaEventRecord(c->tm.ev[0], st));
-  k_gather<<<(c->nsup + 255) / 256, 256, 0, st>>>(c->nsup, c->d_tg_ptr, c->d_tg_col, c->d_tg_val, x, c->d_xs); ++c->launches;
-  EFIE_CUDA(cudaGetLastError());
+  EFIE_TRY(launch_gather(c, st, 1, one_vec(x, c->d_xs)));
   EFIE_CUDA(cudaEventRecord(c->tm.ev[1], st));
   EFIE_TRY(superspace_apply(c, c->d_xs, c->d_ys, c->d_ysn));
-  k_scatter<<<(c->ndof + 255) / 256, 256, 0, st>>>(c->ndof, c->d_ts_ptr, c->d_ts_col, c->d_ts_val, c->d_ys, c->d_ysn,
-                                                  y); ++c->launches;
-  EFIE_CUDA(cudaGetLastError());
+  EFIE_TRY(launch_scatter(c, st, 1, c->d_ys, c->d_ysn, 0, one_vec(nullptr, y)));
   EFIE_CUDA(cudaEventRecord(c->tm.ev[6], st));
   return EFIE_OK;
 }
 
 efie_status dev_scatter(Ctx *c, const double2 *ys, double2 *y) {
-  k_scatter<<<(c->ndof + 255) / 256, 256, 0, c->stream>>>(c->ndof, c->d_ts_ptr, c->d_ts_col, c->d_ts_val, ys, nullptr,
-                                                         y); ++c->launches;
-  EFIE_CUDA(cudaGetLastError());
-  return EFIE_OK;
+  return launch_scatter(c, c->stream, 1, ys, nullptr, 0, one_vec(nullptr, y));
 }
 
-efie_status dev_gather(Ctx *c, const double2 *x, double2 *xs) {
-  k_gather<<<(c->nsup + 255) / 256, 256, 0, c->stream>>>(c->nsup, c->d_tg_ptr, c->d_tg_col, c->d_tg_val, x, xs); ++c->launches;
-  EFIE_CUDA(cudaGetLastError());
-  return EFIE_OK;
+efie_status dev_gather(Ctx *c, const double2 *x, double2 *xs) { return launch_gather(c, c->stream, 1, one_vec(x, xs)); }
+
+__global__ void k_to_f32(size_t n, const double *__restrict__ a, float *__restrict__ b) {
+  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) b[i] = (float)a[i];
 }
 
 efie_status dev_alloc_work(Ctx *c) {
@@ -1242,8 +935,23 @@ efie_status dev_alloc_work(Ctx *c) {
   EFIE_CUDA(cudaMemcpyAsync(c->d_M, c->tab.M.data(), 8 * c->tab.M.size(), cudaMemcpyHostToDevice, c->stream));
   EFIE_CUDA(cudaMemcpyAsync(c->d_Md, c->tab.Md.data(), 8 * c->tab.Md.size(), cudaMemcpyHostToDevice, c->stream));
   EFIE_CUDA(cudaMemcpyAsync(c->d_E, c->tab.E.data(), 8 * c->tab.E.size(), cudaMemcpyHostToDevice, c->stream));
+  if (c->opt.precision == EFIE_MIXED_FP32) {  // the same in FP32, and the tangents at the nodes
+    const size_t nD = ncl * nI * 6;
+    EFIE_TRY(dalloc(c, &c->d_Mf, c->q1 * c->p1));
+    EFIE_TRY(dalloc(c, &c->d_Mdf, c->q1 * c->p1));
+    EFIE_TRY(dalloc(c, &c->d_Ef, 2 * c->q1 * c->q1));
+    EFIE_TRY(dalloc(c, &c->d_nodeDf, nD));
+    auto conv = [&](size_t n, const double *a, float *b) {
+      k_to_f32<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(n, a, b);
+      ++c->launches;
+    };
+    conv(c->q1 * c->p1, c->d_M, c->d_Mf);
+    conv(c->q1 * c->p1, c->d_Md, c->d_Mdf);
+    conv(2 * c->q1 * c->q1, c->d_E, c->d_Ef);
+    conv(nD, c->d_nodeD, c->d_nodeDf);
+    EFIE_CUDA(cudaGetLastError());
+  }
   EFIE_CUDA(cudaStreamSynchronize(c->stream));
-  EFIE_TRY(dev_set_kernel_attrs(c));
   return m2l_store_matrices(c);
 }
 
@@ -1261,57 +969,9 @@ constexpr int kFB = 4 * kRB;       // fields per M2L block
 constexpr int kMultiThreads = 256;
 constexpr int kMultiMaxNI = 144;   // (q + 1)^2 limit of the shared-memory tile
 
-// node-major folded sources of all right-hand sides: src[(id nI + m) ld + 4 r + {x, y, z, div}].
-// The row stride ld = 4 x (allocated right-hand sides) does not change with R, so rows of
-// clusters that receive no M2L stay zero whatever the number of right-hand sides of earlier
-// products.
-__global__ void k_fold_multi(long long tot, int nI, int R, int ld, size_t mstride, const double *__restrict__ nodeD,
-                             const float2 *__restrict__ mom, float2 *__restrict__ src) {
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= tot) return;
-  const int id = (int)(t / nI), mi = (int)(t % nI);
-  const double *D = nodeD + 6 * t;
-  for (int r = 0; r < R; ++r) {
-    const float2 *mm = mom + r * mstride + (size_t)id * 3 * nI;
-    float2 m0 = mm[mi], m1 = mm[nI + mi], nu = mm[2 * nI + mi];
-    float2 *o = src + (size_t)t * ld + 4 * r;
-    for (int k = 0; k < 3; ++k) {
-      float d1 = (float)D[k], d2 = (float)D[3 + k];
-      o[k] = make_float2(d1 * m0.x + d2 * m1.x, d1 * m0.y + d2 * m1.y);
-    }
-    o[3] = nu;
-  }
-}
-
-__global__ void k_unfold_multi(long long tot, int nI, int R, int ld, size_t lstride, float ik2,
-                               const double *__restrict__ nodeD, const float2 *__restrict__ acc,
-                               const float2 *__restrict__ more, int nslab, size_t slab, float2 *__restrict__ loc) {
-  long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= tot) return;
-  const int id = (int)(t / nI), mi = (int)(t % nI);
-  const double *D = nodeD + 6 * t;
-  for (int r = 0; r < R; ++r) {
-    float2 a[4];
-    for (int k = 0; k < 4; ++k) {
-      a[k] = acc[(size_t)t * ld + 4 * r + k];
-      for (int j = 1; j < nslab; ++j) {
-        const float2 b = more[(j - 1) * slab + (size_t)t * (4 * kMmaMaxRhs) + 4 * r + k];
-        a[k] = make_float2(a[k].x + b.x, a[k].y + b.y);
-      }
-    }
-    float l0x = 0, l0y = 0, l1x = 0, l1y = 0;
-    for (int k = 0; k < 3; ++k) {
-      l0x += (float)D[k] * a[k].x;
-      l0y += (float)D[k] * a[k].y;
-      l1x += (float)D[3 + k] * a[k].x;
-      l1y += (float)D[3 + k] * a[k].y;
-    }
-    float2 *l = loc + r * lstride + (size_t)id * 3 * nI;
-    l[mi] = make_float2(l0x, l0y);
-    l[nI + mi] = make_float2(l1x, l1y);
-    l[2 * nI + mi] = make_float2(-ik2 * a[3].x, -ik2 * a[3].y);
-  }
-}
+// Sources and results of all right-hand sides are node-major, src[(id nI + m) ld + 4 r + {x, y, z, div}];
+// the row stride ld = 4 x (allocated right-hand sides) does not change with R, so rows of clusters that
+// receive no M2L stay zero whatever the number of right-hand sides of earlier products.
 
 // One block per (target cluster, group of kRB right-hand sides).  Thread t owns field
 // f = t % kFB of the group and the target nodes m = t / kFB + 8 k.  For every source cluster:
@@ -1453,17 +1113,18 @@ efie_status dev_matvec_batch(Ctx *c, int R, const double2 *const *X, double2 *co
   // phase events as in the single-vector product: 0 start, 1 gathered, 2 near done (second
   // stream), 3 moments folded, 4 M2L done, 5 local expansions evaluated, 6 end
   EFIE_CUDA(cudaEventRecord(c->tm.ev[0], st));
-  const int nI = c->nI, q1 = c->q1, p1 = c->p1, m = c->m;
-  const float h = (float)(1.0 / c->n);
-  const size_t mstride = (size_t)c->ncl * 3 * nI;
-  for (int r = 0; r < R; ++r) {
-    double2 *xs = c->d_xsB + (size_t)r * c->nsup;
-    if (superspace) {
-      EFIE_CUDA(cudaMemcpyAsync(xs, X[r], sizeof(double2) * c->nsup, cudaMemcpyDeviceToDevice, st));
-    } else {
-      k_gather<<<(c->nsup + 255) / 256, 256, 0, st>>>(c->nsup, c->d_tg_ptr, c->d_tg_col, c->d_tg_val,
-                                                      X[r], xs); ++c->launches;
+  const int nI = c->nI;
+  // up to 64 vectors a launch of T and T^T (callers pass at most 64)
+  for (int r0 = 0; r0 < R; r0 += kTMax) {
+    const int n = std::min(kTMax, R - r0);
+    TVecs V;
+    for (int r = 0; r < n; ++r) {
+      V.in[r] = X[r0 + r];
+      V.out[r] = c->d_xsB + (size_t)(r0 + r) * c->nsup;
+      if (superspace)
+        EFIE_CUDA(cudaMemcpyAsync(V.out[r], V.in[r], sizeof(double2) * c->nsup, cudaMemcpyDeviceToDevice, st));
     }
+    if (!superspace) EFIE_TRY(launch_gather(c, st, n, V));
   }
   EFIE_CUDA(cudaEventRecord(c->tm.ev[1], st));
   EFIE_CUDA(cudaEventRecord(c->fork, st));
@@ -1471,18 +1132,8 @@ efie_status dev_matvec_batch(Ctx *c, int R, const double2 *const *X, double2 *co
   EFIE_TRY(dev_near_apply_batch(c, R, c->d_xsB, c->d_ysnB, (size_t)c->nsup, c->stream2));
   EFIE_CUDA(cudaEventRecord(c->tm.ev[2], c->stream2));
   EFIE_CUDA(cudaEventRecord(c->join, c->stream2));
-  // leaf moments and M2M of all right-hand sides: grid dimension y = right-hand side
-  k_leaf_moments<float><<<dim3(c->nE, R), 128, 0, st>>>(c->nE, c->lev_off[m], p1, q1, h, c->d_M, c->d_Md, c->d_xsB,
-                                                        c->d_momB, (size_t)c->nsup, mstride); ++c->launches;
-  for (int l = m - 1; l >= 0; --l) {
-    int npar = c->np << (2 * l);
-    k_m2m<float><<<dim3(npar, R), 128, m2m_smem(q1, sizeof(float2)), st>>>(npar, c->lev_off[l], c->lev_off[l + 1], q1,
-                                                                           c->d_E, c->d_momB, mstride); ++c->launches;
-  }
-  const long long tot = (long long)c->ncl * nI;
-  const unsigned gtot = (unsigned)((tot + 255) / 256);
   const int ld = 4 * c->batch_cap;
-  k_fold_multi<<<gtot, 256, 0, st>>>(tot, nI, R, ld, mstride, c->d_nodeD, c->d_momB, c->d_srcB); ++c->launches;
+  EFIE_TRY(tree_up_f32(c, st, R, c->d_xsB, c->d_momB, c->d_srcB, ld));
   EFIE_CUDA(cudaEventRecord(c->tm.ev[3], st));
   // a few right-hand sides, or tiles too large for tensor memory: kernel entries in mma.sync operands
   // (a lockstep solve keeps the kernel of its first product while systems drop out: the two round
@@ -1515,25 +1166,20 @@ efie_status dev_matvec_batch(Ctx *c, int R, const double2 *const *X, double2 *co
     ++c->launches;
   }
   EFIE_CUDA(cudaEventRecord(c->tm.ev[4], st));
-  k_unfold_multi<<<gtot, 256, 0, st>>>(tot, nI, R, ld, mstride, (float)(1.0 / (c->kappa * c->kappa)), c->d_nodeD,
-                                       c->d_accB, c->d_moreB, nslab, slab, c->d_locB); ++c->launches;
-  for (int l = 0; l < m; ++l) {
-    int npar = c->np << (2 * l);
-    k_l2l<float><<<dim3(npar, R), 128, l2l_smem(q1, sizeof(float2)), st>>>(npar, c->lev_off[l], c->lev_off[l + 1], q1,
-                                                                           c->d_E, c->d_locB, mstride); ++c->launches;
-  }
-  k_leaf_eval<float><<<dim3(c->nE, R), 128, 0, st>>>(c->nE, c->lev_off[m], p1, q1, h, c->d_M, c->d_Md, c->d_locB,
-                                                     c->d_ysB, mstride, (size_t)c->nsup); ++c->launches;
+  EFIE_TRY(tree_down_f32(c, st, R, c->d_accB, ld, c->d_moreB, 4 * kMmaMaxRhs, nslab, slab, c->d_locB, c->d_ysB));
   EFIE_CUDA(cudaEventRecord(c->tm.ev[5], st));
   EFIE_CUDA(cudaStreamWaitEvent(st, c->join, 0));
-  for (int r = 0; r < R; ++r) {
-    if (superspace) {
+  if (superspace) {
+    for (int r = 0; r < R; ++r) {
       k_sum2<<<(c->nsup + 255) / 256, 256, 0, st>>>((size_t)c->nsup, c->d_ysB + (size_t)r * c->nsup,
                                                     c->d_ysnB + (size_t)r * c->nsup, Y[r]); ++c->launches;
-    } else {
-      k_scatter<<<(c->ndof + 255) / 256, 256, 0, st>>>(c->ndof, c->d_ts_ptr, c->d_ts_col, c->d_ts_val,
-                                                       c->d_ysB + (size_t)r * c->nsup,
-                                                       c->d_ysnB + (size_t)r * c->nsup, Y[r]); ++c->launches;
+    }
+  } else {
+    for (int r0 = 0; r0 < R; r0 += kTMax) {
+      const int n = std::min(kTMax, R - r0);
+      TVecs V;
+      for (int r = 0; r < n; ++r) V.out[r] = Y[r0 + r];
+      EFIE_TRY(launch_scatter(c, st, n, c->d_ysB + (size_t)r0 * c->nsup, c->d_ysnB + (size_t)r0 * c->nsup, c->nsup, V));
     }
   }
   EFIE_CUDA(cudaEventRecord(c->tm.ev[6], st));

@@ -205,45 +205,6 @@ __global__ void __launch_bounds__(128) k_K_digits(int ncl, const int *__restrict
   }
 }
 
-// Folded source fields (as k_fold) and the largest |Re|, |Im| of each field on every level (bit
-// patterns of non-negative doubles order as integers; infinities and NaN come out above all).
-__global__ void k_fold_max(int nI, int m, LevOff L, const double *__restrict__ nodeD, const double2 *__restrict__ mom,
-                           double2 *__restrict__ src, unsigned long long *__restrict__ smax) {
-  __shared__ unsigned long long red[4][4];
-  const int id = blockIdx.x;
-  const double2 *mm = mom + (size_t)id * 3 * nI;
-  double2 *s = src + (size_t)id * 4 * nI;
-  unsigned long long big[4] = {0, 0, 0, 0};
-  auto note = [&](int f, double2 v) {
-    const unsigned long long a = __double_as_longlong(fabs(v.x)), b = __double_as_longlong(fabs(v.y));
-    big[f] = max(big[f], max(a, b));
-  };
-  for (int i = threadIdx.x; i < nI; i += blockDim.x) {
-    const double *D = nodeD + 6 * ((size_t)id * nI + i);
-    const double2 m0 = mm[i], m1 = mm[nI + i], nu = mm[2 * nI + i];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const double2 v = make_double2(D[k] * m0.x + D[3 + k] * m1.x, D[k] * m0.y + D[3 + k] * m1.y);
-      s[k * nI + i] = v;
-      note(k, v);
-    }
-    s[3 * nI + i] = nu;
-    note(3, nu);
-  }
-#pragma unroll
-  for (int f = 0; f < 4; ++f) {
-    for (int o = 16; o > 0; o >>= 1) big[f] = max(big[f], __shfl_xor_sync(0xffffffffu, big[f], o));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][f] = big[f];
-  }
-  __syncthreads();
-  if (threadIdx.x < 4) {
-    unsigned long long v = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v = max(v, red[w][threadIdx.x]);
-    unsigned long long *o = smax + 4 * level_of(L, m, id) + threadIdx.x;
-    if (v > *reinterpret_cast<volatile unsigned long long *>(o)) atomicMax(o, v);
-  }
-}
-
 // exponent e with 2^e above v (bit pattern); v = 0: any
 __device__ __forceinline__ int max_exponent(unsigned long long v) { return (int)(v >> 52) - 1022; }
 
@@ -285,21 +246,32 @@ __global__ void __launch_bounds__(MAXT, MINB) k_m2l_f64_digits(
     for (int i = 0; i < 4; ++i) nx[i] = ld_stream(Kt + (size_t)(4 * c0) * step + 32 * i);
   for (int c = c0; c < c1; ++c) {
     __syncthreads();
-    for (int n = threadIdx.x; n < 8 * kF64Nodes; n += blockDim.x) {
-      const int node = n >> 3, col = n & 7, J = c * kF64Nodes + node;
-      unsigned long long u = kOffset;
-      if (J < total) {
-        const int k = J / nIe, i = J - k * nIe;
-        if (i < nI) u = fx[((size_t)fsrc[k0 + k] * nI + i) * 8 + col];
-      }
-      const int kk = node & 15, q = (kk & 7) >> 1, at = kk >> 3;
-      __half *r = reinterpret_cast<__half *>(&sB[node >> 4][0][0][4 * col + q]) + 2 * at + (kk & 1);
-      __half *s = reinterpret_cast<__half *>(&sB[node >> 4][1][0][4 * (col ^ 1) + q]) + 2 * at + (kk & 1);
+    // four (node, column) a thread at a time, their loads in flight together
+    for (int n0 = threadIdx.x; n0 < 8 * kF64Nodes; n0 += 4 * blockDim.x) {
+      unsigned long long u4[4];
 #pragma unroll
-      for (int d = 0; d < 6; ++d) {  // digit 5 - d: vector d / 2, words 2 (d % 2) + {0, 1}
-        const float v = (float)((int)((u >> (50 - 10 * d)) & 1023) - 512);
-        r[(d >> 1) * 256 + 4 * (d & 1)] = __float2half_rn(v);
-        s[(d >> 1) * 256 + 4 * (d & 1)] = __float2half_rn((col & 1) ? -v : v);
+      for (int v = 0; v < 4; ++v) {
+        const int n = n0 + v * blockDim.x, J = c * kF64Nodes + (n >> 3);
+        u4[v] = kOffset;
+        if (n < 8 * kF64Nodes && J < total) {
+          const int k = J / nIe, i = J - k * nIe;
+          if (i < nI) u4[v] = fx[((size_t)fsrc[k0 + k] * nI + i) * 8 + (n & 7)];
+        }
+      }
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        const int n = n0 + v * blockDim.x, node = n >> 3, col = n & 7;
+        if (n >= 8 * kF64Nodes) continue;
+        const unsigned long long u = u4[v];
+        const int kk = node & 15, q = (kk & 7) >> 1, at = kk >> 3;
+        __half *r = reinterpret_cast<__half *>(&sB[node >> 4][0][0][4 * col + q]) + 2 * at + (kk & 1);
+        __half *s = reinterpret_cast<__half *>(&sB[node >> 4][1][0][4 * (col ^ 1) + q]) + 2 * at + (kk & 1);
+#pragma unroll
+        for (int d = 0; d < 6; ++d) {  // digit 5 - d: vector d / 2, words 2 (d % 2) + {0, 1}
+          const float w = (float)((int)((u >> (50 - 10 * d)) & 1023) - 512);
+          r[(d >> 1) * 256 + 4 * (d & 1)] = __float2half_rn(w);
+          s[(d >> 1) * 256 + 4 * (d & 1)] = __float2half_rn((col & 1) ? -w : w);
+        }
       }
     }
     __syncthreads();
@@ -404,10 +376,8 @@ efie_status m2l_f64_digits_build(Ctx *c) {
   return EFIE_OK;
 }
 
-// moments -> folded sources -> d_acc (and d_accmore: c->f64_split partial results)
-efie_status m2l_f64_digits_fold(Ctx *c, cudaStream_t st, const double2 *mom, double2 *src) {
-  EFIE_CUDA(cudaMemsetAsync(c->d_smax, 0, 32 * (size_t)(c->m + 1), st));
-  k_fold_max<<<c->ncl, 128, 0, st>>>(c->nI, c->m, lev_off(c), c->d_nodeD, mom, src, c->d_smax); ++c->launches;
+// fixed-point sources from the folded ones and their largest values per level (d_smax)
+efie_status m2l_f64_digits_fix(Ctx *c, cudaStream_t st, const double2 *src) {
   const long long tot = (long long)c->ncl * c->nI * 4;
   k_src_fix<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(tot, c->nI, c->m, lev_off(c), src, c->d_smax,
                                                            reinterpret_cast<ulonglong2 *>(c->d_fix)); ++c->launches;

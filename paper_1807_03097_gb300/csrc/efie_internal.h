@@ -134,6 +134,7 @@ struct Ctx {
   int lockstep = 0;  // systems of the lockstep solve under way: its products keep one M2L kernel
   double2 *d_xB = nullptr, *d_yB = nullptr, *d_xsB = nullptr, *d_ysB = nullptr, *d_ysnB = nullptr;
   float2 *d_momB = nullptr, *d_srcB = nullptr, *d_accB = nullptr, *d_locB = nullptr;
+  float2 *d_xfB = nullptr;    // x* of a batch in FP32 for the near field
   float2 *d_moreB = nullptr;  // [m2l_split - 1][ncl][nI][4 kMmaMaxRhs]: further splits of d_accB
   int *d_tc_err = nullptr;   // set by a tensor-core M2L whose pipeline wait ran out
   int *d_near_ptr = nullptr, *d_near_src = nullptr;  // CSR by target element

@@ -1077,6 +1077,7 @@ efie_status dev_batch_alloc(Ctx *c, int R) {
   EFIE_TRY(dalloc(c, &c->d_xsB, (size_t)R * c->nsup));
   EFIE_TRY(dalloc(c, &c->d_ysB, (size_t)R * c->nsup));
   EFIE_TRY(dalloc(c, &c->d_ysnB, (size_t)R * c->nsup));
+  if (c->d_nblkf) EFIE_TRY(dalloc(c, &c->d_xfB, (size_t)((R + 3) / 4 * 4) * c->nsup * (c->nb == 8 ? 2 : 1)));
   EFIE_TRY(dalloc(c, &c->d_momB, (size_t)R * ncl * 3 * nI));
   EFIE_TRY(dalloc(c, &c->d_srcB, (size_t)R * ncl * 4 * nI));
   EFIE_TRY(dalloc(c, &c->d_accB, (size_t)R * ncl * 4 * nI));

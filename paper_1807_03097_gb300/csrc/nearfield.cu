@@ -877,115 +877,256 @@ __global__ void __launch_bounds__(128) k_near_apply_8(int nE, int per, const int
   }
 }
 
-// The same product for several right-hand sides (FP32 blocks, mixed form): each block is read
-// once for a group of up to RB right-hand sides (grid dimension y), which divides the HBM
-// traffic of the near field by RB.  Vectors of right-hand side r start at r * vstride.
-template <int NB, int RB>
-__global__ void __launch_bounds__(32 * kApplyWarps) k_near_apply_multi(int nE, int R, size_t vstride,
-                                                                       const int *__restrict__ ptr,
-                                                                       const int *__restrict__ src,
-                                                                       const float2 *__restrict__ blocks,
-                                                                       const double2 *__restrict__ xs,
-                                                                       double2 *__restrict__ ysn) {
-  constexpr int GS = NB <= 8 ? 8 : (NB <= 16 ? 16 : 32);
-  constexpr int NG = 32 / GS;
-  constexpr int RPL = (NB + GS - 1) / GS;
-  constexpr int XPL = (NB + GS - 1) / GS;
-  __shared__ float red[kApplyWarps * NG][NB][RB][2];
-  const int e = blockIdx.x;
-  if (e >= nE) return;
-  const int r0 = blockIdx.y * RB, nr = min(RB, R - r0);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int g = lane / GS, rl = lane % GS;
-  const int gid = warp * NG + g, ngroups = kApplyWarps * NG;
-  float ar[RPL][RB], ai[RPL][RB], cr[RPL][RB], ci[RPL][RB];
-#pragma unroll
-  for (int t = 0; t < RPL; ++t)
-#pragma unroll
-    for (int j = 0; j < RB; ++j) ar[t][j] = ai[t][j] = cr[t][j] = ci[t][j] = 0.f;
-  const int k0 = ptr[e], k1 = ptr[e + 1];
-  for (int kb = k0; kb < k1; kb += ngroups) {
-    const int k = kb + gid;
-    const bool act = k < k1;
-    const float2 *B = blocks + (size_t)(act ? k : k0) * NB * NB;
-    const size_t xo = (size_t)src[act ? k : k0] * NB;
-    float xr[RB][XPL], xi[RB][XPL];
-#pragma unroll
-    for (int j = 0; j < RB; ++j)
-#pragma unroll
-      for (int t = 0; t < XPL; ++t) {
-        const int cidx = rl + GS * t;
-        double2 v = (act && cidx < NB && j < nr) ? xs[(size_t)(r0 + j) * vstride + xo + cidx] : make_double2(0.0, 0.0);
-        xr[j][t] = (float)v.x;
-        xi[j][t] = (float)v.y;
-      }
-    float pr[RPL][RB], pim[RPL][RB];
-#pragma unroll
-    for (int t = 0; t < RPL; ++t)
-#pragma unroll
-      for (int j = 0; j < RB; ++j) pr[t][j] = pim[t][j] = 0.f;
-#pragma unroll
-    for (int tc = 0; tc < XPL; ++tc) {
-      const int ncol = (NB - GS * tc) < GS ? (NB - GS * tc) : GS;
-#pragma unroll 2
-      for (int c0 = 0; c0 < ncol; ++c0) {
-        const int cc = GS * tc + c0;
-        float2 b[RPL];
-#pragma unroll
-        for (int t = 0; t < RPL; ++t) {
-          const int rr = rl + GS * t;
-          if (NB == 8) {  // row pairs: Re, Re, Im, Im
-            const float *v = reinterpret_cast<const float *>(B + cc * NB + (rr & ~1)) + (rr & 1);
-            b[t] = act ? make_float2(v[0], v[2]) : make_float2(0.f, 0.f);
-          } else {
-            b[t] = (act && rr < NB) ? B[cc * NB + rr] : make_float2(0.f, 0.f);
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < RB; ++j) {
-          const float vr = __shfl_sync(0xffffffffu, xr[j][tc], g * GS + c0);
-          const float vi = __shfl_sync(0xffffffffu, xi[j][tc], g * GS + c0);
-#pragma unroll
-          for (int t = 0; t < RPL; ++t) {
-            pr[t][j] += b[t].x * vr - b[t].y * vi;
-            pim[t][j] += b[t].x * vi + b[t].y * vr;
-          }
-        }
-      }
-    }
-    // per-source partial sums enter the running sums with two-sum compensation
-#pragma unroll
-    for (int t = 0; t < RPL; ++t)
-#pragma unroll
-      for (int j = 0; j < RB; ++j) {
-        const float sr = ar[t][j] + pr[t][j], si = ai[t][j] + pim[t][j];
-        const float br = sr - ar[t][j], bi = si - ai[t][j];
-        cr[t][j] += (ar[t][j] - (sr - br)) + (pr[t][j] - br);
-        ci[t][j] += (ai[t][j] - (si - bi)) + (pim[t][j] - bi);
-        ar[t][j] = sr;
-        ai[t][j] = si;
-      }
-  }
-#pragma unroll
-  for (int t = 0; t < RPL; ++t) {
-    const int rr = rl + GS * t;
-    if (rr < NB)
-#pragma unroll
-      for (int j = 0; j < RB; ++j) {
-        red[gid][rr][j][0] = ar[t][j] + cr[t][j];
-        red[gid][rr][j][1] = ai[t][j] + ci[t][j];
-      }
+// x* of several right-hand sides in FP32, the right-hand side fastest: y[i Rp + r] (Rp = R rounded up to 4,
+// zero beyond R), r-th vector at x + r vstride.  HL: with the rounding errors, (Re, Im, Re lo, Im lo).
+template <bool HL>
+__global__ void __launch_bounds__(256) k_vecs_to_f32(int n, int R, int Rp, size_t vstride, const double2 *__restrict__ x,
+                                                     float2 *__restrict__ y) {
+  __shared__ double2 tile[32][33];
+  const int i0 = blockIdx.x * 32, r0 = blockIdx.y * 32, nr = min(32, Rp - r0);
+  for (int r = threadIdx.x >> 5; r < nr; r += 8) {
+    const int i = i0 + (threadIdx.x & 31);
+    tile[r][threadIdx.x & 31] = (i < n && r0 + r < R) ? x[(size_t)(r0 + r) * vstride + i] : make_double2(0.0, 0.0);
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < NB * nr; i += blockDim.x) {
-    const int rr = i % NB, j = i / NB;
-    double sr = 0.0, si = 0.0;
-    for (int q = 0; q < ngroups; ++q) {
-      sr += (double)red[q][rr][j][0];
-      si += (double)red[q][rr][j][1];
-    }
-    ysn[(size_t)(r0 + j) * vstride + (size_t)e * NB + rr] = make_double2(sr, si);
+  for (int k = threadIdx.x; k < 32 * nr; k += 256) {
+    const int r = k % nr, i = k / nr;
+    if (i0 + i >= n) continue;
+    const double2 v = tile[r][i];
+    const float2 h = make_float2((float)v.x, (float)v.y);
+    const size_t o = (size_t)(i0 + i) * Rp + r0 + r;
+    if (HL)
+      reinterpret_cast<float4 *>(y)[o] =
+          make_float4(h.x, h.y, (float)(v.x - (double)h.x), (float)(v.y - (double)h.y));
+    else
+      y[o] = h;
   }
+}
+
+// The lane groups of the product with several right-hand sides: a group of NB / 2 lanes takes one source
+// block and 4 right-hand sides, a lane two of the rows.  NQ groups of a block of 4 warps take different
+// right-hand sides (grid dimension y: the next 4 NQ), the KS = groups / NQ others different sources.
+template <int NB>
+struct NearGroups {
+  static constexpr int RP = NB / 2, Q = 32 / RP, NG = 4 * Q;
+  int gid, rp, ks, KS, quad;
+  bool act;
+  __device__ NearGroups(int R, int NQ) {
+    const int lane = threadIdx.x & 31, lg = lane / RP;
+    rp = lane % RP;
+    gid = (threadIdx.x >> 5) * Q + lg;
+    KS = NG / NQ;
+    ks = gid / NQ;
+    quad = blockIdx.y * NQ + gid % NQ;
+    act = lg < Q && ks < KS && 4 * quad < R;
+  }
+};
+
+// y[right-hand side][row 2 rp: Re, Im; row 2 rp + 1: Re, Im] of a lane to ysn, over the KS sources in a fixed
+// order; red: double [16][NG RP] in shared memory, of which nothing else is in use
+template <int NB>
+__device__ __forceinline__ void near_store(const NearGroups<NB> &G, int R, int NQ, size_t vstride, const double (&y)[4][4],
+                                           double *red, double2 *__restrict__ ysn) {
+  constexpr int RP = NB / 2, W = NearGroups<NB>::NG * RP;
+  const int e = blockIdx.x;
+  if (G.KS > 1) {
+    if (G.act)
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) red[(4 * j + v) * W + G.gid * RP + G.rp] = y[j][v];
+    __syncthreads();
+    for (int o = threadIdx.x; o < NQ * 4 * NB; o += blockDim.x) {
+      const int row = o % NB, j = (o / NB) & 3, qd = o / (4 * NB), r = 4 * (blockIdx.y * NQ + qd) + j;
+      if (r >= R) continue;
+      const double *a = red + (4 * j + 2 * (row & 1)) * W + qd * RP + (row >> 1);
+      double sr = 0.0, si = 0.0;
+      for (int q = 0; q < G.KS; ++q) {
+        sr += a[q * NQ * RP];
+        si += a[W + q * NQ * RP];
+      }
+      ysn[(size_t)r * vstride + (size_t)e * NB + row] = make_double2(sr, si);
+    }
+  } else if (G.act) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (4 * G.quad + j >= R) break;
+      double2 *o = ysn + (size_t)(4 * G.quad + j) * vstride + (size_t)e * NB + 2 * G.rp;
+      o[0] = make_double2(y[j][0], y[j][1]);
+      o[1] = make_double2(y[j][2], y[j][3]);
+    }
+  }
+}
+
+// 8 x 8 blocks, several right-hand sides: every rounding error kept, as in k_near_apply_8 (in plain FP32 sums
+// the lockstep solves of a low frequency met the same noise as the single one).  6 144 elements, 5 right-hand
+// sides, inside the product: 53 -> 70 us, beside an M2L of 1 ms.
+__global__ void __launch_bounds__(128) k_near_apply_8_multi(int nE, int R, int Rp, int NQ, size_t vstride,
+                                                            const int *__restrict__ ptr, const int *__restrict__ src,
+                                                            const float4 *__restrict__ blocks,
+                                                            const float4 *__restrict__ xf, double2 *__restrict__ ysn) {
+  constexpr int NB = 8, RP = 4;
+  __shared__ double red[16 * NearGroups<NB>::NG * RP];
+  const NearGroups<NB> G(R, NQ);
+  const int k1 = G.act ? ptr[blockIdx.x + 1] : 0, nr = min(4, R - 4 * G.quad);
+  const float2 zero = make_float2(0.f, 0.f);
+  float2 hr[4], lr[4], hi[4], li[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) hr[j] = lr[j] = hi[j] = li[j] = zero;
+  for (int k = G.act ? ptr[blockIdx.x] + G.ks : 0; k < k1; k += G.KS) {
+    const float4 *B = blocks + (size_t)k * NB * RP + G.rp;
+    const float4 *X = xf + (size_t)src[k] * NB * Rp + 4 * G.quad;
+    float4 b[NB];
+#pragma unroll
+    for (int c = 0; c < NB; ++c) b[c] = B[c * RP];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (j >= nr) break;
+      float4 x[NB];
+#pragma unroll
+      for (int c = 0; c < NB; ++c) x[c] = X[c * Rp + j];
+#pragma unroll
+      for (int c = 0; c < NB; ++c) {
+        const float2 xr = make_float2(x[c].x, x[c].x), xi = make_float2(x[c].y, x[c].y);
+        const float2 xrl = make_float2(x[c].z, x[c].z), xil = make_float2(x[c].w, x[c].w);
+        const float2 br = make_float2(b[c].x, b[c].y), bi = make_float2(b[c].z, b[c].w);
+        const float2 nb = make_float2(-bi.x, -bi.y);
+        acc_exact(hr[j], lr[j], br, xr, xrl);
+        acc_exact(hi[j], li[j], br, xi, xil);
+        acc_exact(hr[j], lr[j], nb, xi, xil);
+        acc_exact(hi[j], li[j], bi, xr, xrl);
+      }
+    }
+  }
+  double y[4][4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    y[j][0] = (double)hr[j].x + (double)lr[j].x;
+    y[j][1] = (double)hi[j].x + (double)li[j].x;
+    y[j][2] = (double)hr[j].y + (double)lr[j].y;
+    y[j][3] = (double)hi[j].y + (double)li[j].y;
+  }
+  near_store<NB>(G, R, NQ, vstride, y, red, ysn);
+}
+
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Shared memory of one step: KS blocks, then their x* [KS][NB][4 NQ] (bytes)
+template <int NB>
+__host__ __device__ constexpr size_t near_step_bytes(int NQ) {
+  return (size_t)(32 / (NB / 2) * 4 / NQ) * ((size_t)NB * NB * 8 + (size_t)NB * NQ * 32);
+}
+
+// Larger blocks: a step copies KS source blocks and their x* (FP32, the right-hand side fastest) to shared
+// memory with cp.async, S steps deep; per column a lane reads its two rows with one 16-byte load, the
+// 4 entries of x* with two (the same addresses for the group), and does 32 FMA.  A block's partial sums enter the
+// running sums with two-sum compensation.
+// Bound by issue at many right-hand sides (64 of them, 1 024 elements, 32 x 32 blocks: FMA pipe 57 %,
+// shared memory 44 %), by HBM at few.  A thread a row, with x* converted from FP64 and shuffled in
+// every lane for 8 right-hand sides, took 2.0 ms there, this kernel with its loads straight from global memory
+// the same (their latency), with the copies 0.66 ms; inside the product, beside the moments: 5 right-hand
+// sides, 18 x 18: 0.25 -> 0.11 ms; 8, 50 x 50, 384 elements: 0.17 -> 0.13 ms.
+template <int NB, int S>
+__global__ void __launch_bounds__(128) k_near_apply_multi(int nE, int R, int Rp, int NQ, size_t vstride,
+                                                          const int *__restrict__ ptr, const int *__restrict__ src,
+                                                          const float2 *__restrict__ blocks, const float2 *__restrict__ xf,
+                                                          double2 *__restrict__ ysn) {
+  constexpr int RP = NB / 2, NB2 = NB * NB;
+  extern __shared__ float4 nsm[];
+  const NearGroups<NB> G(R, NQ);
+  const int k0 = ptr[blockIdx.x], k1 = ptr[blockIdx.x + 1], KS = G.KS;
+  const int steps = (k1 - k0 + KS - 1) / KS;
+  const int w = 4 * NQ, wv = min(w, Rp - (int)blockIdx.y * w);  // right-hand sides of a row of x*, valid ones
+  const size_t step_f2 = (size_t)KS * (NB2 + NB * w);
+  auto fetch = [&](int s) {
+    if (s < steps) {
+      float2 *sb = reinterpret_cast<float2 *>(nsm) + (s % S) * step_f2, *sx = sb + KS * NB2;
+      const int ka = k0 + s * KS, nk = min(KS, k1 - ka);
+      const float2 *B = blocks + (size_t)ka * NB2;
+      for (int i = 2 * threadIdx.x; i < nk * NB2; i += 256) cp_async16(sb + i, B + i);
+      for (int q = 0; q < nk; ++q) {
+        const float2 *X = xf + (size_t)src[ka + q] * NB * Rp + blockIdx.y * w;
+        for (int i = threadIdx.x; i < NB * wv / 2; i += 128) {
+          const int c = i / (wv / 2), r = 2 * (i - c * (wv / 2));
+          cp_async16(sx + (q * NB + c) * w + r, X + (size_t)c * Rp + r);
+        }
+      }
+    }
+    cp_commit();
+  };
+#pragma unroll
+  for (int s = 0; s < S - 1; ++s) fetch(s);
+  float h[4][4], cmp[4][4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int v = 0; v < 4; ++v) h[j][v] = cmp[j][v] = 0.f;
+  for (int s = 0; s < steps; ++s) {
+    cp_wait<S - 2>();
+    __syncthreads();
+    fetch(s + S - 1);  // into the slot that every warp has left
+    if (!G.act || k0 + s * KS + G.ks >= k1) continue;
+    const float2 *sb = reinterpret_cast<const float2 *>(nsm) + (s % S) * step_f2;
+    const float4 *B = reinterpret_cast<const float4 *>(sb + G.ks * NB2) + G.rp;
+    const float4 *X = reinterpret_cast<const float4 *>(sb + KS * NB2 + (size_t)G.ks * NB * w + 4 * (G.gid % NQ));
+    float p[4][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) p[j][v] = 0.f;
+#pragma unroll 2
+    for (int c = 0; c < NB; ++c) {
+      const float4 b = B[c * RP];
+      const float4 xa = X[c * (w / 2)], xb = X[c * (w / 2) + 1];
+      const float2 x[4] = {make_float2(xa.x, xa.y), make_float2(xa.z, xa.w), make_float2(xb.x, xb.y),
+                           make_float2(xb.z, xb.w)};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        p[j][0] = fmaf(b.x, x[j].x, fmaf(-b.y, x[j].y, p[j][0]));
+        p[j][1] = fmaf(b.x, x[j].y, fmaf(b.y, x[j].x, p[j][1]));
+        p[j][2] = fmaf(b.z, x[j].x, fmaf(-b.w, x[j].y, p[j][2]));
+        p[j][3] = fmaf(b.z, x[j].y, fmaf(b.w, x[j].x, p[j][3]));
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) two_sum(h[j][v], cmp[j][v], p[j][v]);
+  }
+  double y[4][4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+#pragma unroll
+    for (int v = 0; v < 4; ++v) y[j][v] = (double)h[j][v] + (double)cmp[j][v];
+  __syncthreads();  // the steps' memory takes the sums
+  near_store<NB>(G, R, NQ, vstride, y, reinterpret_cast<double *>(nsm), ysn);
+}
+
+template <int NB, int S>
+static efie_status launch_near_multi_s(Ctx *c, int R, int Rp, int nq, size_t vstride, size_t smem, double2 *ysn,
+                                       cudaStream_t st) {
+  EFIE_CUDA(cudaFuncSetAttribute(k_near_apply_multi<NB, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  k_near_apply_multi<NB, S><<<dim3(c->nE, (Rp / 4 + nq - 1) / nq), 128, smem, st>>>(
+      c->nE, R, Rp, nq, vstride, c->d_near_ptr, c->d_near_src, c->d_nblkf, c->d_xfB, ysn);
+  return EFIE_OK;
+}
+
+// Three steps in flight while they stay small enough for three blocks on an SM, else two
+template <int NB>
+static efie_status launch_near_multi(Ctx *c, int R, int Rp, size_t vstride, double2 *ysn, cudaStream_t st) {
+  const int nq = std::min(Rp / 4, NearGroups<NB>::NG);
+  const size_t step = near_step_bytes<NB>(nq), red = sizeof(double) * 16 * NearGroups<NB>::NG * (NB / 2);
+  if (3 * step <= 72 * 1024)
+    return launch_near_multi_s<NB, 3>(c, R, Rp, nq, vstride, std::max(3 * step, red), ysn, st);
+  return launch_near_multi_s<NB, 2>(c, R, Rp, nq, vstride, std::max(2 * step, red), ysn, st);
 }
 
 __global__ void k_blocks_to_f32(size_t n, const double2 *__restrict__ in, float2 *__restrict__ out) {
@@ -1018,24 +1159,26 @@ efie_status dev_near_apply(Ctx *c, const double2 *xs, double2 *ysn, cudaStream_t
 
 // R right-hand sides, vector r at xs + r vstride (FP32 blocks of the mixed form)
 efie_status dev_near_apply_batch(Ctx *c, int R, const double2 *xs, double2 *ysn, size_t vstride, cudaStream_t st) {
-  constexpr int RB = 8;
   if (!c->d_nblkf) {
     for (int r = 0; r < R; ++r) EFIE_TRY(dev_near_apply(c, xs + r * vstride, ysn + r * vstride, st));
     return EFIE_OK;
   }
-  const dim3 grid(c->nE, (R + RB - 1) / RB);
-  const int threads = 32 * kApplyWarps;
+  const int Rp = (R + 3) / 4 * 4;
+  const dim3 gx((c->nsup + 31) / 32, (Rp + 31) / 32);
+  if (c->nb == 8) k_vecs_to_f32<true><<<gx, 256, 0, st>>>(c->nsup, R, Rp, vstride, xs, c->d_xfB);
+  else k_vecs_to_f32<false><<<gx, 256, 0, st>>>(c->nsup, R, Rp, vstride, xs, c->d_xfB);
+  ++c->launches;
   switch (c->nb) {
-#define EFIE_APPLYB_CASE(NBV)                                                                                \
-  case NBV:                                                                                                  \
-    k_near_apply_multi<NBV, RB><<<grid, threads, 0, st>>>(c->nE, R, vstride, c->d_near_ptr, c->d_near_src,   \
-                                                          c->d_nblkf, xs, ysn);                              \
-    break;
-    EFIE_APPLYB_CASE(8)
-    EFIE_APPLYB_CASE(18)
-    EFIE_APPLYB_CASE(32)
-    EFIE_APPLYB_CASE(50)
-#undef EFIE_APPLYB_CASE
+    case 8: {
+      const int nq = std::min(Rp / 4, NearGroups<8>::NG);
+      k_near_apply_8_multi<<<dim3(c->nE, (Rp / 4 + nq - 1) / nq), 128, 0, st>>>(
+          c->nE, R, Rp, nq, vstride, c->d_near_ptr, c->d_near_src, reinterpret_cast<const float4 *>(c->d_nblkf),
+          reinterpret_cast<const float4 *>(c->d_xfB), ysn);
+      break;
+    }
+    case 18: EFIE_TRY(launch_near_multi<18>(c, R, Rp, vstride, ysn, st)); break;
+    case 32: EFIE_TRY(launch_near_multi<32>(c, R, Rp, vstride, ysn, st)); break;
+    case 50: EFIE_TRY(launch_near_multi<50>(c, R, Rp, vstride, ysn, st)); break;
     default:
       c->err = "unsupported block size";
       return EFIE_EINVAL;
@@ -1072,16 +1215,17 @@ efie_status dev_near_apply(Ctx *c, const double2 *xs, double2 *ysn, cudaStream_t
       EFIE_CUDA(cudaGetLastError());
       return EFIE_OK;
     }
+    if (c->nb == 50) {
+      k_near_apply<float, 50><<<c->nE, threads, 0, st>>>(c->nE, c->d_near_ptr, c->d_near_src, c->d_nblkf, xs, ysn);
+      ++c->launches;
+      EFIE_CUDA(cudaGetLastError());
+      return EFIE_OK;
+    }
   }
   switch (c->nb) {
 #define EFIE_APPLY_CASE(NBV)                                                                                   \
   case NBV:                                                                                                   \
-    if (f32)                                                                                                  \
-      k_near_apply<float, NBV><<<c->nE, threads, 0, st>>>(c->nE, c->d_near_ptr, c->d_near_src, c->d_nblkf, xs, \
-                                                          ysn);                                              \
-    else                                                                                                      \
-      k_near_apply<double, NBV><<<c->nE, threads, 0, st>>>(c->nE, c->d_near_ptr, c->d_near_src, c->d_nblk, xs, \
-                                                           ysn);                                             \
+    k_near_apply<double, NBV><<<c->nE, threads, 0, st>>>(c->nE, c->d_near_ptr, c->d_near_src, c->d_nblk, xs, ysn); \
     break;
     EFIE_APPLY_CASE(8)
     EFIE_APPLY_CASE(18)

@@ -94,9 +94,9 @@ __global__ void k_mufu(int iters, float *sink) {
   if (s == 1234.5f) sink[0] = s;
 }
 
-__device__ __forceinline__ void mma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+__device__ __forceinline__ void mma_tf32(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
   asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-               "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d), "l"(a), "l"(b), "r"(idesc),
+               "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d), "l"(a), "l"(b), "r"(idesc),
                "r"(acc)
                : "memory");
 }
@@ -122,22 +122,22 @@ __global__ void k_mma(int N, int iters, long long *cyc, int *err) {
   tc::fence_after_sync();
   const uint32_t tb = *tslot;
   if (warp == 0 && lane == 0) {
-    // bf16 instruction descriptor: FP32 accumulator, A and B bf16 (format 1), K-major
-    const uint32_t idesc = KIND == 0 ? tc::idesc_tf32(128, N)
-                                     : ((1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | (8u << 24));
+    // instruction descriptor: FP32 accumulator, A and B K-major, both TF32 (format 2) or both bf16 (1)
+    const uint32_t fmt = KIND == 0 ? 2u : 1u;
+    const uint32_t idesc = tc::idesc_f16(128, N) | (fmt << 7) | (fmt << 10);
     const uint32_t a0 = tc::smem_u32(smem), b0 = a0 + 64 * 1024;
     uint64_t da[4], db[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      da[k] = tc::smem_desc(a0 + 256 * k);
-      db[k] = tc::smem_desc(b0 + 256 * k);
+      da[k] = tc::smem_desc(a0 + 256 * k, 128, 1024);
+      db[k] = tc::smem_desc(b0 + 256 * k, 128, 1024);
     }
     const long long t0 = clock64();
     for (int i = 0; i < iters; i += 8) {
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
-        if (KIND == 0) tc::mma_tf32(tb, da[k & 3], db[k & 3], idesc, 1u);
-        else mma_f16(tb, da[k & 3], db[k & 3], idesc, 1u);
+        if (KIND == 0) mma_tf32(tb, da[k & 3], db[k & 3], idesc, 1u);
+        else tc::mma_f16(tb, da[k & 3], db[k & 3], idesc, 1u);
       }
     }
     tc::mma_commit(tc::smem_u32(bar));

@@ -46,8 +46,7 @@ void release_device(Ctx *c) {
   dfree(c, c->d_w); dfree(c, c->d_r); dfree(c, c->d_b); dfree(c, c->d_sol); dfree(c, c->d_nrm);
   dfree(c, c->d_xB); dfree(c, c->d_yB); dfree(c, c->d_xsB); dfree(c, c->d_ysB); dfree(c, c->d_ysnB);
   dfree(c, c->d_momB); dfree(c, c->d_srcB); dfree(c, c->d_accB); dfree(c, c->d_locB); dfree(c, c->d_moreB);
-  dfree(c, c->d_xfB);
-  dfree(c, c->d_tc_err);
+  dfree(c, c->d_xfB); dfree(c, c->d_tcA); dfree(c, c->d_tcmax); dfree(c, c->d_tc_err);
   c->batch_cap = 0;
   c->kr = 0;
   c->part_cap = 0;
@@ -579,7 +578,7 @@ static efie_status solve_batched(Ctx *c, int nrhs, const double *b, double *x, i
   size_t fr = 0, tot = 0;
   EFIE_CUDA(cudaMemGetInfo(&fr, &tot));
   const size_t per = gmres_batch_bytes_per_system(c) + 32 * N + size_t(56) * c->nsup +
-                     size_t(80) * c->ncl * c->nI;
+                     size_t(80) * c->ncl * c->nI + (m2l_tc_supported(c) ? m2l_tc_bytes(c, 16) / 16 : 0);
   int chunk = (int)std::min<size_t>(64, (size_t)(0.8 * (double)fr) / std::max<size_t>(per, 1));
   if (chunk < 1) {
     c->err = "solve: the Krylov basis of one system does not fit in the free device memory";

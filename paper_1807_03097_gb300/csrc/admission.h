@@ -38,7 +38,10 @@ inline size_t request_footprint(int np, int level_m, int p, int q, int gmres_res
   // cluster): pair geometry and phase, CSR entries, the unordered-pair lists (48 bytes)
   const size_t clusters = ncl * nI * (72 + 14 * 16) + 130 * ncl * 48;
   const size_t vecs = nE * nb * 16 * 6 + ndof * 16 * 8;
-  const size_t batch = lockstep > 1 ? lockstep * (5 * nE * nb * 16 + 14 * ncl * nI * 8 + 4 * ndof * 16) : 0;
+  // with the sources once more as split FP16 (groups of 8 nodes, 16 right-hand sides at a time)
+  const size_t batch = lockstep > 1 ? lockstep * (5 * nE * nb * 16 + 14 * ncl * nI * 8 + 4 * ndof * 16) +
+                                          (lockstep + 15) / 16 * 4096 * ncl * ((nI + 7) / 8)
+                                    : 0;
   const size_t farfield = ndir > 0 ? 48 * size_t(ndir) * nE + 48 * size_t(ndir) + 24 * size_t(ndir) : 0;
   const bool stored = mixed ? m2l_store == 2 : m2l_store != 1;
   // FP64: rows in tiles of 16, an even number of columns

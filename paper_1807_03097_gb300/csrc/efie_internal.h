@@ -136,6 +136,8 @@ struct Ctx {
   float2 *d_momB = nullptr, *d_srcB = nullptr, *d_accB = nullptr, *d_locB = nullptr;
   float2 *d_xfB = nullptr;    // x* of a batch in FP32 for the near field
   float2 *d_moreB = nullptr;  // [m2l_split - 1][ncl][nI][4 kMmaMaxRhs]: further splits of d_accB
+  uint4 *d_tcA = nullptr;      // sources of a batch split for the tensor-core M2L (m2l_tc.cu)
+  unsigned *d_tcmax = nullptr; // largest source of every field (float bits)
   int *d_tc_err = nullptr;   // set by a tensor-core M2L whose pipeline wait ran out
   int *d_near_ptr = nullptr, *d_near_src = nullptr;  // CSR by target element
   double2 *d_nblk = nullptr;  // [nnear][nb (col)][nb (row)]
@@ -249,6 +251,8 @@ struct MmaArgs {
   size_t slab;
 };
 int m2l_mma_splits(const Ctx *c);
+// lengths in units of 1 / kappa in k_m2l_mma and k_m2l_tc (delta is then the phase)
+inline bool m2l_scaled_lengths(const Ctx *c) { return c->m2l_mode != 2 && c->kappa >= 1e-6 && c->kappa <= 1e6; }
 int m2l_mma_rhs(const Ctx *c);  // right-hand sides up to which a batch takes it
 efie_status launch_m2l_mma(Ctx *c, cudaStream_t st, const MmaArgs &A);
 // product stages around the M2L (tree.cu): xs -> sources, M2L results -> ys; `nrhs` vectors nsup apart
@@ -265,7 +269,8 @@ efie_status m2l_f64_digits_fix(Ctx *c, cudaStream_t st, const double2 *src);
 efie_status m2l_f64_digits_apply(Ctx *c, cudaStream_t st);
 // tensor-core M2L of a batch (m2l_tc.cu)
 bool m2l_tc_supported(const Ctx *c);
-efie_status m2l_tc_prepare(Ctx *c);
+efie_status m2l_tc_prepare(Ctx *c, int nrhs);
+size_t m2l_tc_bytes(const Ctx *c, int nrhs);
 efie_status launch_m2l_tc(Ctx *c, cudaStream_t st, int F, int ld, const float2 *src, float2 *acc);
 efie_status m2l_tc_check(Ctx *c);
 efie_status dev_wait_selftest(Ctx *c, long long cycles);

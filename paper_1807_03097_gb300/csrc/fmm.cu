@@ -1088,7 +1088,9 @@ efie_status dev_batch_alloc(Ctx *c, int R) {
     EFIE_CUDA(cudaMemsetAsync(c->d_moreB, 0, sizeof(float2) * more, c->stream));
   }
   EFIE_TRY(dalloc(c, &c->d_locB, (size_t)R * ncl * 3 * nI));
-  if (c->opt.precision == EFIE_MIXED_FP32 && m2l_tc_supported(c)) EFIE_TRY(m2l_tc_prepare(c));
+  // batches that k_m2l_tc takes (dev_matvec_batch): also room for its split sources
+  if (c->opt.precision == EFIE_MIXED_FP32 && m2l_tc_supported(c))
+    EFIE_TRY(m2l_tc_prepare(c, c->opt.m2l_batch != 1 && R > m2l_mma_rhs(c) ? R : 0));
   const int sm = (int)multi_smem(kMultiMaxNI);
   for (auto fn : {k_m2l_f32_multi<1>, k_m2l_f32_multi<2>, k_m2l_f32_multi<4>, k_m2l_f32_multi<8>,
                   k_m2l_f32_multi<12>, k_m2l_f32_multi<16>, k_m2l_f32_multi<18>})

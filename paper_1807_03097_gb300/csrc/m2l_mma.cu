@@ -349,7 +349,7 @@ static efie_status launch_mma_t(Ctx *c, cudaStream_t st, const MmaArgs &A) {
 
 template <int MT, int NR>
 static efie_status launch_mma_m(Ctx *c, cudaStream_t st, const MmaArgs &A) {
-  const bool fast = c->m2l_mode != 2 && c->kappa >= 1e-6 && c->kappa <= 1e6;
+  const bool fast = m2l_scaled_lengths(c);
   return fast ? launch_mma_t<MT, NR, true>(c, st, A) : launch_mma_t<MT, NR, false>(c, st, A);
 }
 
@@ -374,16 +374,16 @@ int m2l_mma_splits(const Ctx *c) {
 }
 
 // A batch takes this kernel while it is faster than k_m2l_tc, whose cost does not change up to 16
-// right-hand sides (N padded to 64, 96 or 128 target nodes, K to 32 source nodes), while this one's
-// grows with them.  Measured (ms, this kernel / k_m2l_tc, sphere of 1 536 elements): 25 nodes, 6
-// right-hand sides 0.64 / 0.88, 8 right-hand sides 0.94 / 0.89; 49 nodes 5: 1.62 / 1.77, 6: 1.66 / 1.78
-// but 8: 2.47 / 1.78; 81 nodes 4: 2.83 / 3.28, 5: 4.32 / 3.30; 121 nodes 3: 4.36 / 5.25, 4: 5.80 / 5.26.
-// 4.1 times the ratio of the padded tiles separates them.
+// right-hand sides, while this one's grows with them.  Measured (ms, this kernel / k_m2l_tc, sphere of
+// 1 536 elements): 16 nodes, 6 right-hand sides 0.31 / 0.38; 25 nodes 6: 0.64 / 0.67; 49 nodes 3: 0.85 / 1.06,
+// 4: 1.23 / 1.06; 81 nodes 2: 1.47 / 1.96, 3: 2.27 / 1.96; 121 nodes 2: 3.02 / 3.42, 3: 4.37 / 3.42.  Per pair
+// k_m2l_tc takes (rows + 94) x source nodes (rows padded to 64, 96 or 128, nodes to 8), this kernel a
+// right-hand side's (rows + 8) x nodes / 1.36 (rows padded to its tiles).
 int m2l_mma_rhs(const Ctx *c) {
   if (!m2l_tc_supported(c)) return 1 << 30;
   const int nI = c->nI, nw = mma_warps(nI), mt = ((nI + 15) / 16 + nw - 1) / nw;
-  const double here = 16.0 * nw * mt * nI, tc = (nI <= 64 ? 64 : (nI <= 96 ? 96 : 128)) * 32.0 * ((nI + 31) / 32);
-  return std::min(kMmaMaxRhs, (int)(4.1 * tc / here));
+  const double here = (16.0 * nw * mt + 8) * nI, tc = ((nI <= 64 ? 64 : (nI <= 96 ? 96 : 128)) + 94.0) * 8 * ((nI + 7) / 8);
+  return std::max(1, std::min(kMmaMaxRhs, (int)(1.36 * tc / here)));
 }
 
 efie_status launch_m2l_mma(Ctx *c, cudaStream_t st, const MmaArgs &A) {

@@ -1,14 +1,10 @@
 // Blackwell (sm_103a) tensor-core building blocks in inline PTX: tensor-memory allocation,
-// tcgen05.mma of kind::tf32 from shared-memory descriptors, completion through mbarriers,
-// and tensor-memory loads for the epilogue.
+// tcgen05.mma of kind::f16 from shared-memory descriptors, bulk copies into shared memory,
+// completion through mbarriers, and tensor-memory loads for the epilogue.
 //
-// Operand layout used throughout (K-major, no swizzle): a tile of R rows (M or N) by 32
-// K-elements of 4 bytes is a grid of core matrices of 8 rows x 16 bytes (128 contiguous
-// bytes each).  Core matrices adjacent in K are 128 bytes apart (leading byte offset), those
-// adjacent in rows are 1024 bytes apart (stride byte offset); element (r, k) sits at byte
-//   (r / 8) * 1024 + (k / 4) * 128 + (r % 8) * 16 + (k % 4) * 4.
-// One MMA consumes K = 8 (two core matrices along K); step k of a tile starts 256 bytes
-// further on.
+// Operand layout used throughout (K-major, no swizzle): a tile of R rows (M or N) is a grid of core
+// matrices of 8 rows x 16 bytes (8 FP16 K-elements; 128 contiguous bytes each).  One MMA consumes
+// K = 16, two core matrices along K.
 //
 // Every wait on an mbarrier is bounded by a clock deadline; a wait that runs out returns
 // false and the caller records the failure instead of spinning forever.
@@ -18,35 +14,26 @@
 namespace efie {
 namespace tc {
 
-constexpr uint32_t kTileK = 32;         // K-elements per staged tile
-constexpr uint32_t kLBO = 128;          // bytes between core matrices along K
-constexpr uint32_t kSBO = 1024;         // bytes between 8-row groups
-constexpr uint32_t kKStepBytes = 256;   // K = 8 tf32 elements
-
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-// byte offset of element (r, k) inside a [R x 32] K-major tile
-__device__ __forceinline__ uint32_t tile_off(uint32_t r, uint32_t k) {
-  return (r >> 3) * kSBO + (k >> 2) * kLBO + (r & 7) * 16 + (k & 3) * 4;
-}
-
-// Shared-memory matrix descriptor (tcgen05 form): start address, leading and stride byte
-// offsets (all >> 4), descriptor version 1 at bit 46, base offset 0, no swizzle.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
+// Shared-memory matrix descriptor (tcgen05 form): start address, leading byte offset (between core
+// matrices adjacent along K) and stride byte offset (between groups of 8 rows), all >> 4, descriptor
+// version 1 at bit 46, base offset 0, no swizzle.
+__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
   uint64_t d = 0;
   d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)((kLBO >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)((kSBO >> 4) & 0x3FFFu) << 32;
+  d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
+  d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
   d |= (uint64_t)1 << 46;
   return d;
 }
 
-// Instruction descriptor of kind::tf32: FP32 accumulator (bits 4-5 = 1), A and B TF32
-// (bits 7-9, 10-12 = 2), both K-major (bits 15, 16 = 0), N >> 3 at bit 17, M >> 4 at bit 24.
-__host__ __device__ constexpr uint32_t idesc_tf32(uint32_t M, uint32_t N) {
-  return (1u << 4) | (2u << 7) | (2u << 10) | ((N >> 3) << 17) | ((M >> 4) << 24);
+// Instruction descriptor of kind::f16: FP32 accumulator (bits 4-5 = 1), A and B FP16 (bits 7-9,
+// 10-12 = 0), both K-major (bits 15, 16 = 0), N >> 3 at bit 17, M >> 4 at bit 24.
+__host__ __device__ constexpr uint32_t idesc_f16(uint32_t M, uint32_t N) {
+  return (1u << 4) | ((N >> 3) << 17) | ((M >> 4) << 24);
 }
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
@@ -55,6 +42,19 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
 
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(bar) : "memory");
+}
+
+// arrive once and expect `bytes` more of bulk copies in this phase
+__device__ __forceinline__ void mbar_arrive_expect(uint32_t bar, uint32_t bytes) {
+  asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n\t}" ::"r"(bar), "r"(bytes)
+               : "memory");
+}
+
+// one thread: `bytes` (a multiple of 16) from global to shared memory, both 16-byte aligned; counted by bar
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src),
+               "r"(bytes), "r"(bar)
+               : "memory");
 }
 
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
@@ -100,12 +100,12 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 
-// one thread: D (+)= A * B, A [M x 8] and B [N x 8] K-major in shared memory
-__device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                         uint32_t accumulate) {
+// one thread: D (+)= A * B, A [M x 16] and B [N x 16] in FP16, K-major in shared memory
+__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                        uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
@@ -114,20 +114,6 @@ __device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t adesc, uint64
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
                : "memory");
-}
-
-// whole warp: 16 consecutive FP32 columns of this warp's 32 lanes (thread i: lane base + i)
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *v) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-      "%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 // whole warp: 8 consecutive FP32 columns of this warp's 32 lanes
@@ -139,16 +125,6 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float *v) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// whole warp: store 8 consecutive FP32 columns of this warp's 32 lanes
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const float *v) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr),
-               "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
-               "r"(__float_as_uint(v[3])), "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])),
-               "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7]))
-               : "memory");
-  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
 // Asynchronous forms: several loads (or stores) in flight, then one wait.  After wait_ld the
@@ -168,14 +144,6 @@ __device__ __forceinline__ void tmem_st8_async(uint32_t taddr, const uint32_t *r
                : "memory");
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-
-// x = hi + lo with hi rounded to TF32 (10 explicit mantissa bits, to nearest with ties away
-// from zero: add half a TF32 unit to the bit pattern, clear the 13 low bits) and lo = x - hi,
-// exact in FP32; the MMA then sees hi and TF32(lo).  Finite inputs far below FLT_MAX only.
-__device__ __forceinline__ void split_tf32(float x, float &hi, float &lo) {
-  hi = __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u);
-  lo = x - hi;
-}
 
 }  // namespace tc
 }  // namespace efie

@@ -141,14 +141,72 @@ __global__ void k_K_exponent(const int *__restrict__ targets, const int *__restr
   if (threadIdx.x == 0) expo[t] = ilogb(1.001 * 0.25 / (M_PI * sqrt((double)red[0]))) + 1;
 }
 
+constexpr int kCircle = 256;  // points e^{2 pi i n / kCircle} of the table
+
+__global__ void k_circle(double2 *tab) {
+  double sn, cs;
+  sincospi(2.0 * threadIdx.x / kCircle, &sn, &cs);
+  tab[threadIdx.x] = make_double2(cs, sn);
+}
+
+// v 2^(kFixBits - e) rounded to an integer (half away from zero), |v| < 2^e, by shifts of v's mantissa
+__device__ __forceinline__ unsigned long long fix_shift(double v, int e) {
+  const long long b = __double_as_longlong(v);
+  const int ex = (int)((b >> 52) & 0x7ff), sh = ex - 1075 + kFixBits - e;
+  const unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | (ex ? 1ull << 52 : 0ull);
+  const unsigned long long u = sh >= 0 ? m << sh : (sh < -60 ? 0ull : (m + (1ull << (-sh - 1))) >> -sh);
+  return (b < 0 ? 0ull - u : u) + kOffset;
+}
+
+// G = e^{i kappa r} / (4 pi r) from r^2 with 30 FP64 operations (the FP64 pipe takes 72 clocks an instruction and
+// scheduler and bounds k_K_digits; with sqrt, division, sincos and conversions to integers the kernel took 55 ms
+// for 62 880 unordered pairs of 81 nodes, assembly of the 1 536-element sphere 121.6 ms, now 95.3).  1 / r: FP32 reciprocal root of the upper 20 mantissa
+// bits, one step of the third-order iteration (relative error 2^-21 -> 2^-60); r = r^2 / r with one Newton
+// correction.  e^{i x}: table lookup and Taylor polynomials of the remainder (Tang's table-driven method): x = n 2 pi
+// / 256 + t, |t| <= 0.0123, two-constant reduction; sin t to t^5, cos t to t^6 (next terms 2^-57, 2^-66).
+__device__ __forceinline__ double2 green(double r2, double kappa, const double2 *__restrict__ tab) {
+  const long long b = __double_as_longlong(r2);
+  const int ex = (int)(b >> 52);  // r2 = m 2^(ex - 1023); even power: f = m 2^odd in [1, 4), r2 = f 4^h
+  if (ex < 200 || ex > 1800) {    // lengths beyond 1e-120 ... 1e120: the library's functions
+    const double r = sqrt(r2), f = 0.25 / (M_PI * r);
+    double sn, cs;
+    sincos(kappa * r, &sn, &cs);
+    return make_double2(f * cs, f * sn);
+  }
+  const int odd = (ex + 1) & 1, h = (ex - 1023 - odd) / 2;
+  const float f = __int_as_float(((127 + odd) << 23) | (int)((b >> 29) & 0x7fffff));
+  const int yb = __float_as_int(rsqrtf(f));  // in (1/2, 1]
+  const double y0 = __longlong_as_double(((long long)((yb >> 23) - 127 + 1023 - h) << 52) | ((long long)(yb & 0x7fffff) << 29));
+  const double t0 = r2 * y0, e = fma(-t0, y0, 1.0);
+  const double y = fma(e * y0, fma(0.375, e, 0.5), y0);  // 1 / r
+  const double ra = r2 * y, r = fma(0.5 * y, fma(-ra, ra, r2), ra);
+  const double x = kappa * r, g = y * (0.25 / M_PI);
+  if (!(x < 1e9)) {
+    double sn, cs;
+    sincos(x, &sn, &cs);
+    return make_double2(g * cs, g * sn);
+  }
+  const double shifter = 6755399441055744.0;  // 1.5 2^52: the integer in the low bits
+  const double ns = fma(x, kCircle / (2.0 * M_PI), shifter), n = ns - shifter;
+  const double p1 = 2.0 * M_PI / kCircle, p2 = 2.4492935982947064e-16 / kCircle;  // 2 pi = fl(2 pi) + 2.449e-16
+  const double t = fma(-n, p2, fma(-n, p1, x));
+  const double2 cs = tab[(int)__double_as_longlong(ns) & (kCircle - 1)];
+  const double t2 = t * t;
+  const double st = fma(t * t2, fma(t2, 1.0 / 120, -1.0 / 6), t);                  // sin t
+  const double ct = t2 * fma(t2, fma(t2, -1.0 / 720, 1.0 / 24), -0.5);             // cos t - 1
+  return make_double2(g * (cs.x + fma(cs.x, ct, -cs.y * st)), g * (cs.y + fma(cs.y, ct, cs.x * st)));
+}
+
 // One block per unordered admissible pair {t, s}: G is symmetric, so every entry is evaluated once
 // and written into both clusters' matrices.  A thread owns 2 x 2 entries (nodes 2 a, 2 a + 1 of t, 2 b,
 // 2 b + 1 of s; the node count padded to an even nIe), i.e. two fragment words of either side.
 __global__ void __launch_bounds__(128) k_K_digits(int ncl, const int *__restrict__ optr, const int *__restrict__ osrc,
                                                   const int *__restrict__ fptr, const int *__restrict__ fsrc,
                                                   const size_t *__restrict__ koff, const int *__restrict__ expo, int nI,
-                                                  double kappa, const double *__restrict__ nodeX, uint4 *__restrict__ K) {
+                                                  double kappa, const double *__restrict__ nodeX,
+                                                  const double2 *__restrict__ circle, uint4 *__restrict__ K) {
   extern __shared__ double sx[];  // [2][nI][3]
+  __shared__ double2 tab[kCircle];
   __shared__ int sh[4];
   const int u = blockIdx.x, tid = threadIdx.x;
   if (tid == 0) {
@@ -162,6 +220,7 @@ __global__ void __launch_bounds__(128) k_K_digits(int ncl, const int *__restrict
   }
   __syncthreads();
   const int cl[2] = {sh[0], sh[1]};
+  for (int i = tid; i < kCircle; i += blockDim.x) tab[i] = circle[i];
   for (int side = 0; side < 2; ++side)
     for (int k = fptr[cl[side]] + tid; k < fptr[cl[side] + 1]; k += blockDim.x)
       if (fsrc[k] == cl[1 - side]) sh[2 + side] = k - fptr[cl[side]];
@@ -178,12 +237,9 @@ __global__ void __launch_bounds__(128) k_K_digits(int ncl, const int *__restrict
       for (int j = 0; j < 2; ++j) {
         const double *x = sx + 3 * min(2 * a + i, nI - 1), *y = sx + 3 * (nI + min(2 * b + j, nI - 1));
         const double dx = x[0] - y[0], dy = x[1] - y[1], dz = x[2] - y[2];
-        const double r = sqrt(dx * dx + dy * dy + dz * dz);
-        double sn, cs;
-        sincos(kappa * r, &sn, &cs);
-        const double f = 0.25 / (M_PI * r);
-        g[i][j][0] = f * cs;
-        g[i][j][1] = f * sn;
+        const double2 v = green(dx * dx + dy * dy + dz * dz, kappa, tab);
+        g[i][j][0] = v.x;
+        g[i][j][1] = v.y;
       }
 #pragma unroll
     for (int side = 0; side < 2; ++side) {
@@ -198,7 +254,7 @@ __global__ void __launch_bounds__(128) k_K_digits(int ncl, const int *__restrict
 #pragma unroll
         for (int part = 0; part < 2; ++part) {
           const double x = side == 0 ? g[i][0][part] : g[0][i][part], y = side == 0 ? g[i][1][part] : g[1][i][part];
-          __stcs(o + part * 128, pack_pair(fix(x, e), fix(y, e)));
+          __stcs(o + part * 128, pack_pair(fix_shift(x, e), fix_shift(y, e)));
         }
       }
     }
@@ -359,9 +415,13 @@ efie_status m2l_f64_digits_build(Ctx *c) {
   EFIE_CUDA(cudaMemcpyAsync(c->d_koff, off.data(), sizeof(size_t) * off.size(), cudaMemcpyHostToDevice, c->stream));
   k_K_exponent<<<c->n_m2l_targets, 128, 0, c->stream>>>(c->d_m2l_targets, c->d_far_ptr, c->d_far_src, c->nI, c->d_center,
                                                        c->d_nodeXf, c->d_kexp); ++c->launches;
+  DevTemp tmp;
+  double2 *circle = nullptr;
+  EFIE_TRY(tmp.get(c, &circle, kCircle));
+  k_circle<<<1, kCircle, 0, c->stream>>>(circle); ++c->launches;
   k_K_digits<<<c->npairs, 128, sizeof(double) * 6 * c->nI, c->stream>>>(
       c->ncl, c->d_own_ptr, c->d_own_src, c->d_far_ptr, c->d_far_src, c->d_koff, c->d_kexp, c->nI, c->kappa, c->d_nodeX,
-      (uint4 *)c->d_K); ++c->launches;
+      circle, (uint4 *)c->d_K); ++c->launches;
   EFIE_CUDA(cudaGetLastError());
   // splits of the K-steps: enough warps for the chip when there are few targets, two staged chunks each
   const long long warps = 16ll * c->nsm, have = (long long)c->n_m2l_targets * ((c->nI + 15) / 16);

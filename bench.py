@@ -413,7 +413,7 @@ def run_gpu(args):
         t64 = time.perf_counter() - t0
         E64, W64 = e64[0].cpu().numpy(), w64[0].cpu().numpy()
         fp64 = {"solves_per_s": 1.0 / t64, "ms_per_solve": t64 * 1e3, "gmres_iterations": int(info64.iterations),
-                "converged": bool(info64.converged), "m2l": "stored FP64 coupling matrices",
+                "converged": bool(info64.converged), "m2l": "kept FP64 coupling matrices (digits, FP16 tensor cores)",
                 "far_field_rel_err_mixed_vs_fp64": float(np.abs(e_mixed - E64).max() / np.abs(E64).max()),
                 "current_rel_err_mixed_vs_fp64": float(np.linalg.norm(w_mixed - W64) / np.linalg.norm(W64)),
                 "note": "far-field error = max over 64 directions and 3 components of |E_mixed - E_fp64|, "
@@ -436,10 +436,10 @@ def run_gpu(args):
             "frac": achieved / fp32_peak, "traffic": None, "peak_note": peak_note,
             "work": f"{n_eval:.3e} kernel entries x {flops_per_eval:.0f} flop per matvec", "m2l_ms": m2l_ms}
     if pk_alu:
-        # time each pipe needs for the entries at its measured rate (per entry: 8 packed FMAs on
-        # the FMA pipe and 3 MUFU operations in the direct-phase form)
+        # time each pipe needs for the entries at its measured rate (per entry: 13 packed
+        # operations on two entries at a time and 3 MUFU operations; the fields are multiplied on the tensor cores)
         mufu_rate = min(pk_alu["rsqrt_per_s"], pk_alu["sin_per_s"], pk_alu["cos_per_s"])
-        roof["pipe_bound_ms"] = {"fma_32flop_per_entry": n_eval * 32 / pk_alu["ffma2_flops"] * 1e3,
+        roof["pipe_bound_ms"] = {"fma_26flop_per_entry": n_eval * 26 / pk_alu["ffma2_flops"] * 1e3,
                                  "mufu_3_per_entry": n_eval * 3 / mufu_rate * 1e3}
     # near-field apply timed alone (efie_near_apply, CUDA events on the library's stream) and, for
     # reference, inside the product where it shares the GPU with the far-field chain
@@ -459,11 +459,12 @@ def run_gpu(args):
                  "peak_note": "MEASURED_PEAKS.json hbm_gbs (copy bandwidth)"}
     near_roof["frac"] = near_roof["achieved"] / near_roof["peak"]
     st_ = {k: statistics.median([x_[k] for x_ in setups]) for k in setups[0]}
-    # k_near_quad: per quadrature point and block entry, the integrand of eq. Vkh is a real
-    # combination of two products (geometry term and div-div term: 2 FMA) scaled by the complex
-    # kernel value (2 FMA): 8 FP64 flop per entry and point
+    # k_near_touch: the direct sum takes per quadrature point and block entry a real combination of two
+    # products (geometry term and div-div term: 2 FMA) scaled by the complex kernel value (2 FMA),
+    # 8 FP64 flop; the kernel sums one direction after the other, so its own count is far lower and
+    # the direct sum's rate says nothing about its use of the pipe
     quad_flop = st_["near_quad_points"] * s.nb * s.nb * 8.0
-    roof_setup = {"kernel": "k_near_quad", "bound": "alu (FP64)", "unit": "TFLOP/s",
+    roof_setup = {"kernel": "k_near_touch", "bound": "alu (FP64)", "unit": "TFLOP/s of the direct sum",
                   "achieved": quad_flop / (st_["near_quad_ms"] * 1e-3) / 1e12, "near_quad_ms": st_["near_quad_ms"],
                   "setup_ms": st_["setup_ms"], "work": f"{st_['near_quad_points']:.3e} quadrature points x "
                                                         f"{s.nb}^2 entries x 8 flop",
@@ -473,8 +474,8 @@ def run_gpu(args):
                           "(element tables), timed separately"}
     if pk_alu:
         roof_setup["peak"] = pk_alu["dfma_flops"] / 1e12
-        roof_setup["frac"] = roof_setup["achieved"] / roof_setup["peak"]
-        roof_setup["peak_note"] = "FP64 DFMA measured on this GPU (microbench/peaks.cu)"
+        roof_setup["peak_note"] = ("FP64 DFMA measured on this GPU (microbench/peaks.cu); achieved above it: sum "
+                                   "factorisation (fewer flop for the same sums)")
 
     # end to end through the C ABI with host buffers (copies inside the timed region)
     deg, ncp, knots, cp, wgt = flatten(geo)
@@ -628,7 +629,7 @@ MULTI = {
     "p": 3, "elements_per_patch": "64x64", "level_m": 6, "kappa": 20.0, "q": 10, "eta": 1.6,
     "rhs": 64, "directions": "plane waves, directions normalised Gaussian, polarisation random unit vector "
                              "orthogonal to the direction, seed 1807",
-    "precision": "mixed: M2L split-TF32 on the tensor cores with FP32 accumulation, near field FP32 blocks "
+    "precision": "mixed: M2L split-FP16 on the tensor cores with FP32 accumulation, near field FP32 blocks "
                  "from FP64 quadrature, geometry FP64",
     "l2": "working set > L2 (near-field blocks 19 GB FP32, 64 x 2.1e6 superspace vectors)",
 }
@@ -697,33 +698,25 @@ def multi_leg(args, steps=None, pk_alu=None):
             fp64["single_fp32"].append(float(torch.linalg.norm(y1 - y64) / n64))
         fp64["fp64_matvec_ms"] = s64.last_timings()["total"]
         s64.close()
-    # roofline of the tensor-core M2L (useful complex work; TF32 peak = measured BF16 peak x
-    # the nominal TF32/BF16 ratio 1.1/2.25)
+    # roofline of the tensor-core M2L (useful complex work against the FP16 / BF16 dense rate)
     pk = peaks()
     nI = (w["q"] + 1) ** 2
     useful = 8.0 * nI * nI * 4 * R * s.nfar
     np_ = 64 if nI <= 64 else (96 if nI <= 96 else 128)
-    kp = 8 * sum(min(4, (nI - 32 * c + 7) // 8) for c in range((nI + 31) // 32))
+    kp = 8 * ((nI + 7) // 8)
     executed = 3 * 2.0 * 128 * (2 * np_) * kp * ((4 * R + 63) // 64) * s.nfar
-    tf32_peak = pk.get("bf16_tflops", 1900.0) * 1.1 / 2.25
+    f16_peak = pk.get("bf16_tflops", 1900.0)
     m2l_s = mv["m2l"] * 1e-3
-    roof = {"kernel": "k_m2l_tc", "bound": "tensor", "achieved": useful / m2l_s / 1e12, "peak": tf32_peak,
-            "unit": "TFLOP/s", "frac": useful / m2l_s / 1e12 / tf32_peak, "traffic": None,
-            "peak_note": "TF32 dense = measured BF16 burst peak x 1.1/2.25 (nominal ratio)",
+    roof = {"kernel": "k_m2l_tc", "bound": "tensor", "achieved": useful / m2l_s / 1e12, "peak": f16_peak,
+            "unit": "TFLOP/s", "frac": useful / m2l_s / 1e12 / f16_peak, "traffic": None,
+            "peak_note": "measured BF16 burst peak (MEASURED_PEAKS.json); FP16 runs at the same rate",
             "work": f"useful 8 n_I^2 x 4R x far pairs = {useful:.3e} real flop per product "
-                    f"(complex MACs of {4 * R} fields); executed on the tensor pipe (3 split-TF32 passes, "
+                    f"(complex MACs of {4 * R} fields); executed on the tensor pipe (3 split-FP16 passes, "
                     f"padded to N={2 * np_}, K={kp}) = {executed:.3e}",
-            "executed_tflops": executed / m2l_s / 1e12, "m2l_ms": mv["m2l"]}
-    if pk_alu and pk_alu.get("tcgen05_tf32_flops", 0) > 0:
-        # the primary peak: tcgen05 TF32 as measured on this GPU (microbench/peaks.cu); the
-        # BF16-derived figure stays beside it
-        tf = pk_alu["tcgen05_tf32_flops"] / 1e12
-        roof["peak_derived_bf16x1.1/2.25"] = tf32_peak
-        roof["frac_of_derived_peak"] = roof["frac"]
-        roof["peak"] = tf
-        roof["frac"] = useful / m2l_s / 1e12 / tf
-        roof["peak_note"] = "tcgen05.mma kind::tf32 (M128 N256) measured on this GPU (microbench/peaks.cu)"
-        roof["executed_frac"] = executed / m2l_s / 1e12 / tf
+            "executed_tflops": executed / m2l_s / 1e12, "executed_frac": executed / m2l_s / 1e12 / f16_peak,
+            "m2l_ms": mv["m2l"]}
+    if pk_alu and pk_alu.get("tcgen05_bf16_flops", 0) > 0:
+        roof["frac_of_tcgen05_bf16_measured"] = useful / m2l_s / pk_alu["tcgen05_bf16_flops"]
     # end to end with host buffers
     yh = np.empty_like(b)
     torch.cuda.synchronize()
@@ -735,7 +728,7 @@ def multi_leg(args, steps=None, pk_alu=None):
                       "batched product), mixed precision",
             "value": R * 1000.0 / ms, "unit": "matvec/s", "n_gpus": 1, "steps": steps, "warmup": args.warmup,
             "ms_per_step": ms, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-            "dtype": "tf32x3-m2l/f32/f64", "data": "synthetic", "config": MULTI, "ndof": int(N),
+            "dtype": "f16x3-m2l/f32/f64", "data": "synthetic", "config": MULTI, "ndof": int(N),
             "far_pairs": int(s.nfar), "near_pairs": int(s.nnear), "setup_s": setup_s,
             "matvec_ms_phases": mv, "single_rhs_matvec_ms": single_ms,
             "tensor_vs_single_rhs_rel_diff": diffs, "rel_err_vs_fp64": fp64, "roofline": roof, "cpu_baseline": None,

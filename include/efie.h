@@ -53,8 +53,10 @@ typedef int efie_status;
 
 #define EFIE_FP64 0           /* every step in FP64 */
 #define EFIE_MIXED_FP32 1     /* moments, M2M, M2L, L2L in FP32 (phase split, FP64 per-pair
-                                 phase); the near-field blocks are integrated in FP64 and
-                                 applied from an FP32 copy with compensated FP32 sums;
+                                 phase; products on the tensor cores from FP32 operands split into
+                                 two TF32 or FP16 parts); the near-field blocks are integrated in FP64
+                                 and applied from an FP32 copy with compensated FP32 sums (p = 1: every
+                                 rounding error of the product kept);
                                  geometry, right-hand side, far field and GMRES in FP64 */
 
 #define EFIE_PTR_HOST 0
@@ -81,13 +83,15 @@ typedef struct {
   int gmres_maxit;   /* total iteration cap */
   int tol_is_relative; /* 1: ||r|| <= tol ||b||, 0: ||r|| <= tol */
   int m2l_store;     /* M2L coupling matrices: 0 automatic (FP64 form: kept in device memory
-                        when they take at most half of the free memory; FP32 form: evaluated
+                        when they take at most half of the free memory, as fixed-point digits whose
+                        products the tensor cores do exactly; mixed form: evaluated
                         in every product, which is faster than streaming them); 1 always
                         evaluate; 2 always keep (EFIE_ENOMEM if they do not fit) */
   int m2l_batch;     /* M2L of a product with several right-hand sides in the mixed form:
-                        0 automatic (split TF32 on the tensor cores),
-                        1 FP32 on the CUDA cores, 2 tensor cores (split TF32 with FP32
-                        accumulation, q <= 10; EFIE_EINVAL at setup otherwise) */
+                        0 automatic, 1 FP32 on the CUDA cores, 2 tensor cores (q <= 10;
+                        EFIE_EINVAL at setup otherwise).  0 and 2: kernel entries in the operands of
+                        mma.sync (split TF32) for a few right-hand sides and for q > 10, tcgen05
+                        (split FP16) for more, both with FP32 accumulation */
   int leaf_dense;    /* 0: the paper's block tree (Algorithm 1); 1: leaf-level variant, in which
                         an admissible pair of two elements is integrated as an element block
                         (tensor Gauss, quad_regular points) like a separated near pair instead of

@@ -152,8 +152,8 @@ void drop_product_graph(Ctx *c) {
   dfree(c, c->d_mvin);
 }
 
-// The product of the single-system solver as one CUDA-graph launch: the product chain (about
-// 20 small kernels around the M2L, near field on the second stream) is captured once per setup
+// The product of the single-system solver as one CUDA-graph launch: the product chain (the tree's
+// stages around the M2L, near field on the second stream) is captured once per setup
 // with input d_mvin and output d_w, and replayed, without the launch gaps between its kernels.
 static efie_status gmres_product_prepare(Ctx *c) {
   if (c->g_mv) return EFIE_OK;

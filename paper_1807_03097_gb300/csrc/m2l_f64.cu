@@ -159,11 +159,12 @@ __device__ __forceinline__ unsigned long long fix_shift(double v, int e) {
 }
 
 // G = e^{i kappa r} / (4 pi r) from r^2 with 30 FP64 operations (the FP64 pipe takes 72 clocks an instruction and
-// scheduler and bounds k_K_digits; with sqrt, division, sincos and conversions to integers the kernel took 55 ms
-// for 62 880 unordered pairs of 81 nodes, assembly of the 1 536-element sphere 121.6 ms, now 95.3).  1 / r: FP32 reciprocal root of the upper 20 mantissa
-// bits, one step of the third-order iteration (relative error 2^-21 -> 2^-60); r = r^2 / r with one Newton
-// correction.  e^{i x}: table lookup and Taylor polynomials of the remainder (Tang's table-driven method): x = n 2 pi
-// / 256 + t, |t| <= 0.0123, two-constant reduction; sin t to t^5, cos t to t^6 (next terms 2^-57, 2^-66).
+// scheduler and bounds k_K_digits; with sqrt, division, sincos and conversions to integers the kernel took
+// 55 ms for 62 880 unordered pairs of 81 nodes, now 29; assembly of the 1 536-element sphere 121.6 -> 95.3 ms).
+// 1 / r: FP32 reciprocal root of the upper 23 mantissa bits, one step of the third-order iteration (relative error
+// 2^-21 -> 2^-60); r = r^2 / r with one Newton correction.  e^{i x}: table lookup and Taylor polynomials of the
+// remainder (Tang's table-driven method): x = n 2 pi / 256 + t, |t| <= 0.0123, two-constant reduction; sin t to
+// t^5, cos t to t^6 (next terms 2^-57, 2^-66).
 __device__ __forceinline__ double2 green(double r2, double kappa, const double2 *__restrict__ tab) {
   const long long b = __double_as_longlong(r2);
   const int ex = (int)(b >> 52);  // r2 = m 2^(ex - 1023); even power: f = m 2^odd in [1, 4), r2 = f 4^h

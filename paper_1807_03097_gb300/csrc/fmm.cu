@@ -1071,6 +1071,7 @@ static size_t multi_smem(int nI) {
 
 efie_status dev_batch_alloc(Ctx *c, int R) {
   if (R <= c->batch_cap) return EFIE_OK;
+  c->batch_cap = 0;  // should an allocation fail, the next product allocates all of them again
   const size_t ncl = c->ncl, nI = c->nI;
   EFIE_TRY(dalloc(c, &c->d_xB, (size_t)R * c->ndof));
   EFIE_TRY(dalloc(c, &c->d_yB, (size_t)R * c->ndof));

@@ -28,7 +28,9 @@
 // tensor pipe is busy, which an evaluating warp cannot afford.  Shared memory holds four stages of 4
 // groups of 8 source nodes; the groups of all sources follow one another without padding to whole
 // stages.  Stages are handed over with mbarriers; every wait is bounded and a wait that runs out
-// sets an error flag for the host.
+// sets an error flag for the host.  The copy lane and the MMA lane then issue nothing more and wait, with a
+// fresh bound, for what they have in flight, so that the block neither reuses nor leaves its memory under
+// a copy or an MMA.
 //
 // Bound: shared memory (a stage of 32 nodes at 121 target nodes: 1 740 clocks, of which the MMAs read 580, their
 // pipe is busy 770, the A copies take 130 and the loads and stores of the evaluation 650) and the latency of
@@ -39,6 +41,7 @@
 // 64 bits 2.3e-6 -> 1.3e-6.
 #include "efie_internal.h"
 #include "tc.cuh"
+#include "tc_pipeline.h"
 #include "fastmath.cuh"
 #include <cuda_fp16.h>
 #include <type_traits>
@@ -216,10 +219,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_m2l_tc(
   extern __shared__ __align__(1024) uint8_t smem[];
   float4 *sC = reinterpret_cast<float4 *>(smem + L::kConst);
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L::kBars);
-  uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 3 * kTcStages + 2);
+  uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 3 * kTcStages + 3);
   int *sRmin = reinterpret_cast<int *>(tslot + 1);
   const uint32_t b_full = tc::smem_u32(&bars[0]), b_empty = tc::smem_u32(&bars[kTcStages]);
-  const uint32_t b_const = tc::smem_u32(&bars[2 * kTcStages + 2]);
+  const uint32_t b_const = tc::smem_u32(&bars[2 * kTcStages + 2]), b_done = tc::smem_u32(&bars[3 * kTcStages + 2]);
   const uint32_t b_tfull = tc::smem_u32(&bars[2 * kTcStages]), b_tempty = tc::smem_u32(&bars[2 * kTcStages + 1]);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int t = targets[blockIdx.x];
@@ -236,6 +239,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_m2l_tc(
     }
     tc::mbar_init(b_tfull, 1);
     tc::mbar_init(b_tempty, kTcProducers);
+    tc::mbar_init(b_done, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     *sRmin = 0x7f7fffff;
   }
@@ -262,9 +266,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_m2l_tc(
   const uint32_t tq = tbase + ((uint32_t)(32 * q) << 16);
   long long patience = kTcWaitCycles;  // of this thread's waits; none after one has run out
   auto wait = [&](uint32_t bar, uint32_t parity, int code) {
-    if (tc::mbar_wait(bar, parity, patience)) return;
+    if (tc::mbar_wait(bar, parity, patience)) return true;
     atomicOr(err, code);
     patience = 0;
+    return false;
   };
 
   if (warp < kTcWarps) {
@@ -354,47 +359,62 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_m2l_tc(
     const uint64_t dah0 = tc::smem_desc(a0, 2 * L::kA, 128), dal0 = tc::smem_desc(a0 + L::kA, 2 * L::kA, 128);
     const uint64_t dbh0 = tc::smem_desc(a0 + L::kOffB, 2 * L::kB, 128);
     const uint64_t dbl0 = tc::smem_desc(a0 + L::kOffB + L::kB, 2 * L::kB, 128);
-    for (int it = 0, c = 0, g = 0; it < T; ++it) {
-      const int st = it % kTcStages;
-      // [D1 D2] (+)= A [Re B; Im B]^T, three split products per K-step
-      if (c == 0 && it > 0) wait(b_tempty, g++ & 1, 4);
-      wait(b_full + 8 * st, (it / kTcStages) & 1, 8);
-      tc::fence_after_sync();
+    int c = 0, g = 0;  // stage of the group, group
+    const int issued = issue_stages(
+        T,
+        [&](int it) {
+          if (c == 0 && it > 0 && !wait(b_tempty, g++ & 1, 4)) return false;
+          return wait(b_full + 8 * (it % kTcStages), (it / kTcStages) & 1, 8);
+        },
+        [&](int it) {
+          // [D1 D2] (+)= A [Re B; Im B]^T, three split products per K-step
+          const int st = it % kTcStages;
+          tc::fence_after_sync();
 #pragma unroll
-      for (int ks = 0; ks < 2; ++ks) {
-        if (4 * it + 2 * ks >= ngrp) break;
-        const uint64_t oa = (uint64_t)(st * (L::kStage >> 4) + ks * (4 * L::kA >> 4));
-        const uint64_t ob = (uint64_t)(st * (L::kStage >> 4) + ks * (4 * L::kB >> 4));
-        tc::mma_f16(tbase, dah0 + oa, dbh0 + ob, idesc, (c == 0 && ks == 0) ? 0u : 1u);
-        tc::mma_f16(tbase, dah0 + oa, dbl0 + ob, idesc, 1u);
-        tc::mma_f16(tbase, dal0 + oa, dbh0 + ob, idesc, 1u);
-      }
-      tc::mma_commit(b_empty + 8 * st);
-      if (++c == KG) c = 0;
-      if (c == 0 || it == T - 1) tc::mma_commit(b_tfull);
-    }
+          for (int ks = 0; ks < 2; ++ks) {
+            if (4 * it + 2 * ks >= ngrp) break;
+            const uint64_t oa = (uint64_t)(st * (L::kStage >> 4) + ks * (4 * L::kA >> 4));
+            const uint64_t ob = (uint64_t)(st * (L::kStage >> 4) + ks * (4 * L::kB >> 4));
+            tc::mma_f16(tbase, dah0 + oa, dbh0 + ob, idesc, (c == 0 && ks == 0) ? 0u : 1u);
+            tc::mma_f16(tbase, dah0 + oa, dbl0 + ob, idesc, 1u);
+            tc::mma_f16(tbase, dal0 + oa, dbh0 + ob, idesc, 1u);
+          }
+          tc::mma_commit(b_empty + 8 * st);
+          if (++c == KG) c = 0;
+          if (c == 0 || it == T - 1) tc::mma_commit(b_tfull);
+        });
+    // no MMA is in flight when the block goes on: the last group's completion, or after an early end that of
+    // what was issued
+    if (issued < T) tc::mma_commit(b_done);
+    if (T > 0 && !(issued < T ? tc::mbar_wait(b_done, 0, kTcWaitCycles)
+                              : tc::mbar_wait(b_tfull, ((T - 1) / KG) & 1, kTcWaitCycles)))
+      atomicOr(err, 128);
   } else if (warp == kTcWarps + 1 && lane == 0) {
     // -------------------------------------------------------------- bulk copies of A
     // A stage past the last group repeats it: its B is zero.
     int lp = 0, lc = 0;
     int s = nsrc > 0 ? ldg_pin(fsrc + k0) : 0;
-    for (int it = 0; it < T; ++it) {
-      const int st = it % kTcStages;
-      if (it >= kTcStages) wait(b_empty + 8 * st, ((it / kTcStages) & 1) ^ 1, 32);
-      tc::mbar_arrive_expect(b_full + 8 * st, 4 * 2 * L::kA);
+    const int issued = issue_stages(
+        T, [&](int it) { return it < kTcStages || wait(b_empty + 8 * (it % kTcStages), ((it / kTcStages) & 1) ^ 1, 32); },
+        [&](int it) {
+          const int st = it % kTcStages;
+          tc::mbar_arrive_expect(b_full + 8 * st, 4 * 2 * L::kA);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        tc::bulk_load(tc::smem_u32(smem) + st * L::kStage + i * 2 * L::kA,
-                      opA + (((size_t)s * KG + lc) * gridDim.y + blockIdx.y) * 256, 2 * L::kA, b_full + 8 * st);
-        if (4 * it + i + 1 >= ngrp) continue;
-        if (++lc == KG) {
-          lc = 0;
-          s = ldg_pin(fsrc + k0 + ++lp);
-        }
-      }
-    }
-    // no copy is in flight when the block ends
-    for (int it = max(T - kTcStages, 0); it < T; ++it) wait(b_full + 8 * (it % kTcStages), (it / kTcStages) & 1, 32);
+          for (int i = 0; i < 4; ++i) {
+            tc::bulk_load(tc::smem_u32(smem) + st * L::kStage + i * 2 * L::kA,
+                          opA + (((size_t)s * KG + lc) * gridDim.y + blockIdx.y) * 256, 2 * L::kA, b_full + 8 * st);
+            if (4 * it + i + 1 >= ngrp) continue;
+            if (++lc == KG) {
+              lc = 0;
+              s = ldg_pin(fsrc + k0 + ++lp);
+            }
+          }
+        });
+    // a phase completes only with its copies (it was armed after the one before had completed), and the
+    // evaluating warps arrive in every phase
+    drain_stages(issued, kTcStages, [&](int it) {
+      if (!tc::mbar_wait(b_full + 8 * (it % kTcStages), (it / kTcStages) & 1, kTcWaitCycles)) atomicOr(err, 32);
+    });
   } else if (warp == kTcWarps + 2) {
     // -------------------------------------------------------- source node constants
     // Lane l: node l % 8 of the stage's group l / 8.  Nodes past the pair's or the list's end repeat the
@@ -449,7 +469,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_m2l_tc(
   float *sS1 = reinterpret_cast<float *>(smem), *sS2 = sS1 + 128 * (NP + 1);
   const int m = 32 * q + lane;
   if (warp >= kTcWarps) {
-    // the other two warps take no part in staging the sums
+    // the MMA, copy and constants warps take no part in staging the sums
   } else if (nsrc >= 1) {
     tc::fence_after_sync();
 #pragma unroll 1

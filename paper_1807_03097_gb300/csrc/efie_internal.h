@@ -295,6 +295,21 @@ efie_status dev_gmres_batch(Ctx *c, int R, const double2 *const *b, double2 *con
     if (s_ < 0) return s_;         \
   } while (0)
 
+// Allows a kernel its dynamic shared memory before a launch that takes `bytes` (beyond 48 KB it has to be
+// asked for).  The limit belongs to the function on the device, not to a context, and other host threads
+// launch the same function with other sizes: so the value is a constant of the function, the largest
+// size of its range, and never this launch's.
+template <size_t Limit, class F>
+inline efie_status allow_smem(Ctx *c, F *f, size_t bytes) {
+  static_assert(Limit <= 227 * 1024, "dynamic shared memory of a block");
+  if (bytes > Limit) {
+    c->err = "shared memory of a kernel beyond its range";
+    return EFIE_EINVAL;
+  }
+  if (bytes > 48 * 1024) EFIE_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Limit));
+  return EFIE_OK;
+}
+
 // Device memory (devmem.cpp): stream-ordered allocations on the context's stream from one pool
 // per device, counted per context.  pool_ref / pool_unref bracket the lifetime of a context or
 // a server on a device; pinned_get / pinned_put hand out reusable pinned host buffers.

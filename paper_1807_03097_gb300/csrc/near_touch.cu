@@ -396,12 +396,14 @@ __global__ void __launch_bounds__(TouchCfg<P>::kThreads, P == 2 ? 3 : 1) k_near_
   }
 }
 
+constexpr size_t kTouchSmem = 200 * 1024;  // rules that need more stay with k_near_quad
+
 // Whether this geometry and rule can take the factorised kernel: at most two points a thread, shared
 // memory for one block, and no knot inside an element (every element in one knot span).
 template <int P>
 static bool touch_fits(int g, int gdsel) {
   const size_t d = gdsel == 2 ? touch_smem_doubles<P, 2>(g) : (gdsel == 4 ? touch_smem_doubles<P, 4>(g) : touch_smem_doubles<P, 8>(g));
-  return g <= 16 && g * g * g <= 2 * TouchCfg<P>::kThreads && d * sizeof(double) <= 200 * 1024;
+  return g <= 16 && g * g * g <= 2 * TouchCfg<P>::kThreads && d * sizeof(double) <= kTouchSmem;
 }
 
 bool near_touch_supported(const Ctx *c, int gdsel) {
@@ -422,7 +424,7 @@ bool near_touch_supported(const Ctx *c, int gdsel) {
 template <int P, int GD>
 static efie_status launch_touch(Ctx *c, const TouchArgs &A) {
   const size_t smem = sizeof(double) * touch_smem_doubles<P, GD>(A.g);
-  EFIE_CUDA(cudaFuncSetAttribute(k_near_touch<P, GD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  EFIE_TRY((allow_smem<kTouchSmem>(c, k_near_touch<P, GD>, smem)));
   k_near_touch<P, GD><<<A.ntodo, TouchCfg<P>::kThreads, smem, c->stream>>>(A);
   ++c->launches;
   EFIE_CUDA(cudaGetLastError());

@@ -524,8 +524,7 @@ efie_status dev_near_quadrature(Ctx *c, const std::vector<NearPair> &pairs, cons
 #define EFIE_QUAD(PP, GG)                                                                                 \
   if (!launched && c->p == PP && GDsel == GG) {                                                           \
     const size_t smem = sizeof(double) * quad_smem_doubles<PP>();                                         \
-    EFIE_CUDA(cudaFuncSetAttribute(k_near_quad<PP, GG>, cudaFuncAttributeMaxDynamicSharedMemorySize,     \
-                                   (int)smem));                                                          \
+    EFIE_TRY((allow_smem<sizeof(double) * quad_smem_doubles<PP>()>(c, k_near_quad<PP, GG>, smem)));       \
     k_near_quad<PP, GG><<<A.ntodo, kQuadThreads, smem, c->stream>>>(A);                                   \
     ++c->launches;                                                                                        \
     launched = true;                                                                                      \
@@ -564,7 +563,7 @@ efie_status dev_near_quadrature(Ctx *c, const std::vector<NearPair> &pairs, cons
 #define EFIE_SEP(PP)                                                                                   \
   case PP: {                                                                                           \
     const size_t smem = sep_smem<PP>(g);                                                               \
-    EFIE_CUDA(cudaFuncSetAttribute(k_near_sep<PP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
+    EFIE_TRY((allow_smem<sep_smem<PP>(kSepMaxG)>(c, k_near_sep<PP>, smem)));                           \
     k_near_sep<PP><<<S.nlist, 128, smem, s0>>>(S);                                                     \
     ++c->launches;                                                                                     \
     break;                                                                                             \
@@ -1025,6 +1024,25 @@ __host__ __device__ constexpr size_t near_step_bytes(int NQ) {
   return (size_t)(32 / (NB / 2) * 4 / NQ) * ((size_t)NB * NB * 8 + (size_t)NB * NQ * 32);
 }
 
+// Three steps in flight while they stay small enough for three blocks on an SM, else two.
+template <int NB>
+constexpr int near_steps(int NQ) {
+  return 3 * near_step_bytes<NB>(NQ) <= 72 * 1024 ? 3 : 2;
+}
+// Shared memory of a block (its steps, at the end the sums), and the most that any NQ takes with S steps
+template <int NB>
+constexpr size_t near_smem(int NQ) {
+  const size_t steps = near_steps<NB>(NQ) * near_step_bytes<NB>(NQ), red = sizeof(double) * 16 * NearGroups<NB>::NG * (NB / 2);
+  return steps > red ? steps : red;
+}
+template <int NB, int S>
+constexpr size_t near_smem_limit() {
+  size_t most = 0;
+  for (int nq = 1; nq <= NearGroups<NB>::NG; ++nq)
+    if (near_steps<NB>(nq) == S && near_smem<NB>(nq) > most) most = near_smem<NB>(nq);
+  return most;
+}
+
 // Larger blocks: a step copies KS source blocks and their x* (FP32, the right-hand side fastest) to shared
 // memory with cp.async, S steps deep; per column a lane reads its two rows with one 16-byte load, the
 // 4 entries of x* with two (the same addresses for the group), and does 32 FMA.  A block's partial sums enter the
@@ -1113,20 +1131,17 @@ __global__ void __launch_bounds__(128) k_near_apply_multi(int nE, int R, int Rp,
 template <int NB, int S>
 static efie_status launch_near_multi_s(Ctx *c, int R, int Rp, int nq, size_t vstride, size_t smem, double2 *ysn,
                                        cudaStream_t st) {
-  EFIE_CUDA(cudaFuncSetAttribute(k_near_apply_multi<NB, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  EFIE_TRY((allow_smem<near_smem_limit<NB, S>()>(c, k_near_apply_multi<NB, S>, smem)));
   k_near_apply_multi<NB, S><<<dim3(c->nE, (Rp / 4 + nq - 1) / nq), 128, smem, st>>>(
       c->nE, R, Rp, nq, vstride, c->d_near_ptr, c->d_near_src, c->d_nblkf, c->d_xfB, ysn);
   return EFIE_OK;
 }
 
-// Three steps in flight while they stay small enough for three blocks on an SM, else two
 template <int NB>
 static efie_status launch_near_multi(Ctx *c, int R, int Rp, size_t vstride, double2 *ysn, cudaStream_t st) {
   const int nq = std::min(Rp / 4, NearGroups<NB>::NG);
-  const size_t step = near_step_bytes<NB>(nq), red = sizeof(double) * 16 * NearGroups<NB>::NG * (NB / 2);
-  if (3 * step <= 72 * 1024)
-    return launch_near_multi_s<NB, 3>(c, R, Rp, nq, vstride, std::max(3 * step, red), ysn, st);
-  return launch_near_multi_s<NB, 2>(c, R, Rp, nq, vstride, std::max(2 * step, red), ysn, st);
+  if (near_steps<NB>(nq) == 3) return launch_near_multi_s<NB, 3>(c, R, Rp, nq, vstride, near_smem<NB>(nq), ysn, st);
+  return launch_near_multi_s<NB, 2>(c, R, Rp, nq, vstride, near_smem<NB>(nq), ysn, st);
 }
 
 __global__ void k_blocks_to_f32(size_t n, const double2 *__restrict__ in, float2 *__restrict__ out) {

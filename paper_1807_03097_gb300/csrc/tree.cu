@@ -350,10 +350,16 @@ TreeArgs<double> tree_args(const Ctx *c, const double *D, int ld) {
   return {c->q1, c->p1, c->nI, c->d_M, c->d_Md, c->d_E, D, 1.0 / c->n, 1.0 / (c->kappa * c->kappa), ld};
 }
 
-// dynamic shared memory beyond 48 KB has to be asked for
-template <class F>
-cudaError_t allow_smem(F *f, size_t bytes) {
-  return bytes > 48 * 1024 ? cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) : cudaSuccess;
+// dynamic shared memory of k_up and k_down (leaves: of NC children evaluated in the block); their largest
+// sizes at kMaxQ1, kMaxP1 are the functions' limits
+template <class R>
+constexpr size_t up_smem(int q1) {
+  return sizeof(C2<R>) * 24 * q1 * q1 + sizeof(R) * 2 * q1 * q1;
+}
+template <class R>
+constexpr size_t down_smem(int q1, int p1, int leaves) {
+  const size_t nI = (size_t)q1 * q1;
+  return sizeof(C2<R>) * 9 * nI + sizeof(R) * (2 * nI + 2 * q1 * p1) + leaves * sizeof(C2<R>) * (3 * nI + 4 * q1 * p1);
 }
 
 // Leaves with their parents in one block; not in FP64 while the parents are fewer than the SMs: the FP64
@@ -372,19 +378,19 @@ efie_status up(Ctx *c, cudaStream_t st, int nrhs, const R *D, const double2 *xs,
   const bool fused = leaves_fused<R>(c);
   if (!fused) {
     const size_t sm = up_leaf_smem<R>(c->q1, c->p1, 1);
-    EFIE_CUDA(allow_smem(k_up_leaf<R, 1>, sm));
+    EFIE_TRY((allow_smem<up_leaf_smem<R>(kMaxQ1, kMaxP1, 1)>(c, k_up_leaf<R, 1>, sm)));
     k_up_leaf<R, 1><<<dim3(c->nE, nrhs), kTreeThreads, sm, st>>>(A, c->lev_off[m], 0, xs, xstride, mom, mstride, src, mx(m),
                                                               nullptr);
     ++c->launches;
   } else {
     const size_t sm = up_leaf_smem<R>(c->q1, c->p1, 4);
-    EFIE_CUDA(allow_smem(k_up_leaf<R, 4>, sm));
+    EFIE_TRY((allow_smem<up_leaf_smem<R>(kMaxQ1, kMaxP1, 4)>(c, k_up_leaf<R, 4>, sm)));
     k_up_leaf<R, 4><<<dim3(c->nE / 4, nrhs), kTreeThreads, sm, st>>>(A, c->lev_off[m], c->lev_off[m - 1], xs, xstride, mom,
                                                                   mstride, src, mx(m), mx(m - 1));
     ++c->launches;
   }
-  const size_t sm = sizeof(C2<R>) * 24 * c->nI + sizeof(R) * 2 * c->nI;
-  EFIE_CUDA(allow_smem(k_up<R>, sm));
+  const size_t sm = up_smem<R>(c->q1);
+  EFIE_TRY((allow_smem<up_smem<R>(kMaxQ1)>(c, k_up<R>, sm)));
   for (int l = m - (fused ? 2 : 1); l >= 0; --l) {
     k_up<R><<<dim3(c->np << (2 * l), nrhs), kTreeThreads, sm, st>>>(A, c->lev_off[l], c->lev_off[l + 1], mom, mstride, src, mx(l));
     ++c->launches;
@@ -397,24 +403,25 @@ template <class R>
 efie_status down(Ctx *c, cudaStream_t st, int nrhs, const R *D, int ld, const C2<R> *acc, C2<R> *loc, size_t lstride,
                  double2 *ys, size_t ystride) {
   const TreeArgs<R> A = tree_args(c, D, ld);
-  const int m = c->m, nI = c->nI;
-  const size_t base = sizeof(C2<R>) * 9 * nI + sizeof(R) * (2 * nI + 2 * c->q1 * c->p1);
-  const size_t per = sizeof(C2<R>) * (3 * nI + 4 * c->q1 * c->p1);
+  const int m = c->m;
+  const size_t base = down_smem<R>(c->q1, c->p1, 0);
   const bool fused = leaves_fused<R>(c);
-  EFIE_CUDA(allow_smem((k_down<R, false, 4>), base));
+  EFIE_TRY((allow_smem<down_smem<R>(kMaxQ1, kMaxP1, 0)>(c, k_down<R, false, 4>, base)));
   for (int l = 0; l < m - (fused ? 1 : 0); ++l) {
     k_down<R, false, 4><<<dim3(c->np << (2 * l), nrhs), kTreeThreads, base, st>>>(A, acc, c->lev_off[l], c->lev_off[l + 1],
                                                                                   l == 0, loc, lstride, ys, ystride);
     ++c->launches;
   }
   if (fused) {
-    EFIE_CUDA(allow_smem((k_down<R, true, 4>), base + 4 * per));
-    k_down<R, true, 4><<<dim3(c->nE / 4, nrhs), kTreeThreads, base + 4 * per, st>>>(A, acc, c->lev_off[m - 1], c->lev_off[m],
-                                                                                 m == 1, loc, lstride, ys, ystride);
+    const size_t sm = down_smem<R>(c->q1, c->p1, 4);
+    EFIE_TRY((allow_smem<down_smem<R>(kMaxQ1, kMaxP1, 4)>(c, k_down<R, true, 4>, sm)));
+    k_down<R, true, 4><<<dim3(c->nE / 4, nrhs), kTreeThreads, sm, st>>>(A, acc, c->lev_off[m - 1], c->lev_off[m], m == 1,
+                                                                     loc, lstride, ys, ystride);
   } else {
-    EFIE_CUDA(allow_smem((k_down<R, true, 1>), base + per));
-    k_down<R, true, 1><<<dim3(c->nE, nrhs), kTreeThreads, base + per, st>>>(A, acc, c->lev_off[m], 0, m == 0, loc, lstride,
-                                                                          ys, ystride);
+    const size_t sm = down_smem<R>(c->q1, c->p1, 1);
+    EFIE_TRY((allow_smem<down_smem<R>(kMaxQ1, kMaxP1, 1)>(c, k_down<R, true, 1>, sm)));
+    k_down<R, true, 1><<<dim3(c->nE, nrhs), kTreeThreads, sm, st>>>(A, acc, c->lev_off[m], 0, m == 0, loc, lstride, ys,
+                                                                 ystride);
   }
   ++c->launches;
   EFIE_CUDA(cudaGetLastError());

@@ -1046,7 +1046,8 @@ constexpr size_t near_smem_limit() {
 // Larger blocks: a step copies KS source blocks and their x* (FP32, the right-hand side fastest) to shared
 // memory with cp.async, S steps deep; per column a lane reads its two rows with one 16-byte load, the
 // 4 entries of x* with two (the same addresses for the group), and does 32 FMA.  A block's partial sums enter the
-// running sums with two-sum compensation.
+// running sums with two-sum compensation.  Within a block the two halves of a complex product (b.x x.x and -b.y x.y) run in
+// sums of their own: one sum for both is rounded twice a column, 1.2 times the error of the product.
 // Bound by issue at many right-hand sides (64 of them, 1 024 elements, 32 x 32 blocks: FMA pipe 57 %,
 // shared memory 44 %), by HBM at few.  A thread a row, with x* converted from FP64 and shuffled in
 // every lane for 8 right-hand sides, took 2.0 ms there, this kernel with its loads straight from global memory
@@ -1095,11 +1096,11 @@ __global__ void __launch_bounds__(128) k_near_apply_multi(int nE, int R, int Rp,
     const float2 *sb = reinterpret_cast<const float2 *>(nsm) + (s % S) * step_f2;
     const float4 *B = reinterpret_cast<const float4 *>(sb + G.ks * NB2) + G.rp;
     const float4 *X = reinterpret_cast<const float4 *>(sb + KS * NB2 + (size_t)G.ks * NB * w + 4 * (G.gid % NQ));
-    float p[4][4];
+    float p[4][4], m[4][4];
 #pragma unroll
     for (int j = 0; j < 4; ++j)
 #pragma unroll
-      for (int v = 0; v < 4; ++v) p[j][v] = 0.f;
+      for (int v = 0; v < 4; ++v) p[j][v] = m[j][v] = 0.f;
 #pragma unroll 2
     for (int c = 0; c < NB; ++c) {
       const float4 b = B[c * RP];
@@ -1108,16 +1109,20 @@ __global__ void __launch_bounds__(128) k_near_apply_multi(int nE, int R, int Rp,
                            make_float2(xb.z, xb.w)};
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        p[j][0] = fmaf(b.x, x[j].x, fmaf(-b.y, x[j].y, p[j][0]));
-        p[j][1] = fmaf(b.x, x[j].y, fmaf(b.y, x[j].x, p[j][1]));
-        p[j][2] = fmaf(b.z, x[j].x, fmaf(-b.w, x[j].y, p[j][2]));
-        p[j][3] = fmaf(b.z, x[j].y, fmaf(b.w, x[j].x, p[j][3]));
+        p[j][0] = fmaf(b.x, x[j].x, p[j][0]);
+        m[j][0] = fmaf(-b.y, x[j].y, m[j][0]);
+        p[j][1] = fmaf(b.x, x[j].y, p[j][1]);
+        m[j][1] = fmaf(b.y, x[j].x, m[j][1]);
+        p[j][2] = fmaf(b.z, x[j].x, p[j][2]);
+        m[j][2] = fmaf(-b.w, x[j].y, m[j][2]);
+        p[j][3] = fmaf(b.z, x[j].y, p[j][3]);
+        m[j][3] = fmaf(b.w, x[j].x, m[j][3]);
       }
     }
 #pragma unroll
     for (int j = 0; j < 4; ++j)
 #pragma unroll
-      for (int v = 0; v < 4; ++v) two_sum(h[j][v], cmp[j][v], p[j][v]);
+      for (int v = 0; v < 4; ++v) two_sum(h[j][v], cmp[j][v], p[j][v] + m[j][v]);
   }
   double y[4][4];
 #pragma unroll

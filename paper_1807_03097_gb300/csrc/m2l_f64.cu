@@ -114,31 +114,49 @@ __device__ __forceinline__ void digit_products(float (&D)[7][4], const uint4 (&w
 
 }  // namespace
 
-// exponent e with 2^e >= 1.001 / (4 pi r) for every node distance r of a target's far list (distances
-// in FP32 from offsets to the cluster centres)
+// Exponent e with 2^e >= 1.001 / (4 pi r) for every node distance r of a target's far list.  Distances are taken in
+// FP32 from offsets to the cluster centres (81 nodes: 0.2 of the 29 ms of k_K_digits, which FP64 would take again)
+// and once more in FP64 from the coordinates where FP32 may not resolve them: a centre distance whose square
+// leaves its range, or nodes 1e3 times closer than the centres.  A list with a distance whose square FP64
+// does not hold (or is 0) gets kBadExponent.
+constexpr int kBadExponent = 1 << 20;
 __global__ void k_K_exponent(const int *__restrict__ targets, const int *__restrict__ fptr, const int *__restrict__ fsrc,
                              int nI, const double *__restrict__ center, const float *__restrict__ nodeXf,
-                             int *__restrict__ expo) {
-  __shared__ float red[128];
+                             const double *__restrict__ nodeX, int *__restrict__ expo) {
+  __shared__ double red[128];
   const int t = targets[blockIdx.x];
-  float lo = 3e38f;
+  double least = INFINITY;
   for (int k = fptr[t]; k < fptr[t + 1]; ++k) {
     const int s = fsrc[k];
-    const float d0 = (float)(center[4 * t] - center[4 * s]), d1 = (float)(center[4 * t + 1] - center[4 * s + 1]),
-                d2 = (float)(center[4 * t + 2] - center[4 * s + 2]);
+    const double e0 = center[4 * t] - center[4 * s], e1 = center[4 * t + 1] - center[4 * s + 1],
+                 e2 = center[4 * t + 2] - center[4 * s + 2];
+    const float d0 = (float)e0, d1 = (float)e1, d2 = (float)e2, far = fmaxf(fabsf(d0), fmaxf(fabsf(d1), fabsf(d2)));
+    const bool in_range = far > 0x1p-40f && far < 0x1p40f;
+    float lo = 3e38f;
+    if (in_range)
+      for (int i = threadIdx.x; i < nI * nI; i += blockDim.x) {
+        const float *a = nodeXf + ((size_t)t * nI + i / nI) * 3, *b = nodeXf + ((size_t)s * nI + i % nI) * 3;
+        const float x = d0 + a[0] - b[0], y = d1 + a[1] - b[1], z = d2 + a[2] - b[2];
+        lo = fminf(lo, x * x + y * y + z * z);
+      }
+    if (in_range && lo > 1e-6f * far * far) {
+      least = fmin(least, (double)lo);
+      continue;
+    }
     for (int i = threadIdx.x; i < nI * nI; i += blockDim.x) {
-      const float *a = nodeXf + ((size_t)t * nI + i / nI) * 3, *b = nodeXf + ((size_t)s * nI + i % nI) * 3;
-      const float x = d0 + a[0] - b[0], y = d1 + a[1] - b[1], z = d2 + a[2] - b[2];
-      lo = fminf(lo, x * x + y * y + z * z);
+      const double *a = nodeX + ((size_t)t * nI + i / nI) * 3, *b = nodeX + ((size_t)s * nI + i % nI) * 3;
+      const double x = a[0] - b[0], y = a[1] - b[1], z = a[2] - b[2], r2 = x * x + y * y + z * z;
+      least = r2 < INFINITY ? fmin(least, r2) : 0.0;  // an infinity or NaN: not representable
     }
   }
-  red[threadIdx.x] = lo;
+  red[threadIdx.x] = least;
   __syncthreads();
   for (int s = 64; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) red[threadIdx.x] = fminf(red[threadIdx.x], red[threadIdx.x + s]);
+    if ((int)threadIdx.x < s) red[threadIdx.x] = fmin(red[threadIdx.x], red[threadIdx.x + s]);
     __syncthreads();
   }
-  if (threadIdx.x == 0) expo[t] = ilogb(1.001 * 0.25 / (M_PI * sqrt((double)red[0]))) + 1;
+  if (threadIdx.x == 0)
+    expo[t] = red[0] > 0.0 && red[0] < INFINITY ? ilogb(1.001 * 0.25 / (M_PI * sqrt(red[0]))) + 1 : kBadExponent;
 }
 
 constexpr int kCircle = 256;  // points e^{2 pi i n / kCircle} of the table
@@ -375,7 +393,8 @@ __global__ void __launch_bounds__(MAXT, MINB) k_m2l_f64_digits(
   // accumulator registers: (row g, field q) Re, Im, then (row g + 8, field q)
   const int g = lane >> 2, f = lane & 3, row = 16 * warp + g;
   const unsigned long long big = smax[4 * level_of(L, m, t) + f];
-  const bool bad = (big >> 52) >= 2047;  // an infinity or NaN among the sources of this level
+  // an infinity or NaN among the sources of this level, or a distance without an FP64 square in the list
+  const bool bad = (big >> 52) >= 2047 || expo[t] == kBadExponent;
   const int e = expo[t] + max_exponent(big) - 2 * kFixBits + 80;
   double v[4];
 #pragma unroll
@@ -415,7 +434,7 @@ efie_status m2l_f64_digits_build(Ctx *c) {
   EFIE_TRY(dalloc(c, &c->d_fix, (size_t)c->ncl * c->nI * 8));
   EFIE_CUDA(cudaMemcpyAsync(c->d_koff, off.data(), sizeof(size_t) * off.size(), cudaMemcpyHostToDevice, c->stream));
   k_K_exponent<<<c->n_m2l_targets, 128, 0, c->stream>>>(c->d_m2l_targets, c->d_far_ptr, c->d_far_src, c->nI, c->d_center,
-                                                       c->d_nodeXf, c->d_kexp); ++c->launches;
+                                                       c->d_nodeXf, c->d_nodeX, c->d_kexp); ++c->launches;
   DevTemp tmp;
   double2 *circle = nullptr;
   EFIE_TRY(tmp.get(c, &circle, kCircle));

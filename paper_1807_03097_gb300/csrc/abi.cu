@@ -39,8 +39,7 @@ void release_device(Ctx *c) {
   dfree(c, c->d_own_ptr); dfree(c, c->d_own_src); dfree(c, c->d_own_slot); dfree(c, c->d_own_targets);
   dfree(c, c->d_par_ptr); dfree(c, c->d_par_slot); dfree(c, c->d_red); dfree(c, c->d_own_pgeo);
   dfree(c, c->d_own_pph); dfree(c, c->d_back);
-  dfree(c, c->d_K); dfree(c, c->d_koff); dfree(c, c->d_kexp); dfree(c, c->d_smax); dfree(c, c->d_fix);
-  dfree(c, c->d_accmore);
+  m2l_f64_digits_free(c);
   c->k_stored = c->k_digits = false;
   dfree(c, c->d_V); dfree(c, c->d_H); dfree(c, c->d_h); dfree(c, c->d_h2); dfree(c, c->d_part); dfree(c, c->d_gs);
   dfree(c, c->d_w); dfree(c, c->d_r); dfree(c, c->d_b); dfree(c, c->d_sol); dfree(c, c->d_nrm);

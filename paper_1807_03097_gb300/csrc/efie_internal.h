@@ -264,6 +264,8 @@ efie_status tree_down_f64(Ctx *c, cudaStream_t st, double2 *acc, const double2 *
                           double2 *ys);
 // FP64 M2L from kept matrices in digits on the FP16 tensor cores (m2l_f64.cu)
 size_t m2l_f64_digits_bytes(const Ctx *c);
+size_t m2l_f64_digits_beside(const Ctx *c);  // device memory of the form beside the matrices
+void m2l_f64_digits_free(Ctx *c);            // both
 efie_status m2l_f64_digits_build(Ctx *c);
 efie_status m2l_f64_digits_fix(Ctx *c, cudaStream_t st, const double2 *src);
 efie_status m2l_f64_digits_apply(Ctx *c, cudaStream_t st);

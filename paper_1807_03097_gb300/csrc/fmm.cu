@@ -16,6 +16,7 @@
 #include <cmath>
 
 #include "efie_internal.h"
+#include "kept_matrices.h"
 #include "fastmath.cuh"
 
 namespace efie {
@@ -669,16 +670,19 @@ static efie_status m2l_store_matrices(Ctx *c) {
   // bottleneck of that form on this GPU, while the FP32 form evaluates faster than HBM can
   // stream the stored matrices)
   if (c->opt.m2l_store == 0 && f32) return EFIE_OK;
-  // FP64 form: as digits for the tensor cores (rows padded to 16 target nodes, so 1.2 to 1.3 times the
-  // bytes at q >= 4), else, where only the plain matrices fit, for the FP64 pipe
+  // FP64 form: as digits for the tensor cores (target nodes padded to 16, source nodes to an even count: 4 times the
+  // bytes at q = 1, 1.33 at q = 4 to 6, 1.0 at q = 7, 1.2 at q = 8, 1.07 at q = 10), else, where only the plain
+  // matrices fit, for the FP64 pipe
   if (!f32 && 2 * c->npairs == c->nfar) {
     const size_t digits = m2l_f64_digits_bytes(c);
-    if (digits <= (c->opt.m2l_store == 0 ? freeb / 2 : freeb) && pool_alloc(c, &c->d_K, digits) == EFIE_OK) {
-      EFIE_TRY(m2l_f64_digits_build(c));
-      c->k_stored = c->k_digits = true;
-      return EFIE_OK;
+    if (keep_digits(c->opt.m2l_store, digits, m2l_f64_digits_beside(c), freeb) &&
+        pool_alloc(c, &c->d_K, digits) == EFIE_OK) {
+      const efie_status s = m2l_f64_digits_build(c);
+      c->k_stored = c->k_digits = s == EFIE_OK;
+      if (s != EFIE_ENOMEM) return s;
+      m2l_f64_digits_free(c);
     }
-    c->d_K = nullptr;
+    c->err.clear();
   }
   if (c->opt.m2l_store == 0 && bytes > freeb / 2) return EFIE_OK;
   if (pool_alloc(c, &c->d_K, bytes) != EFIE_OK) {

@@ -421,8 +421,30 @@ static std::vector<size_t> k_steps(const Ctx *c) {
   return off;
 }
 
+// splits of the K-steps: enough warps for the chip when there are few targets, two staged chunks each
+static int k_splits(const Ctx *c, size_t steps) {
+  const long long warps = 16ll * c->nsm, have = (long long)c->n_m2l_targets * ((c->nI + 15) / 16);
+  const long long chunks = (long long)(steps / 4) / std::max(c->n_m2l_targets, 1);
+  return (int)std::max(1ll, std::min({2 * warps / have, chunks / 2, 16ll}));
+}
+
 size_t m2l_f64_digits_bytes(const Ctx *c) {
   return k_steps(c).back() * (size_t)((c->nI + 15) / 16) * 4096;
+}
+
+size_t m2l_f64_digits_beside(const Ctx *c) {
+  const size_t nodes = (size_t)c->ncl * c->nI;
+  return 64 * nodes * k_splits(c, k_steps(c).back()) + 12 * (size_t)(c->ncl + 1) + 32 * (size_t)(c->m + 1) +
+         sizeof(double2) * kCircle;
+}
+
+void m2l_f64_digits_free(Ctx *c) {
+  dfree(c, c->d_K);
+  dfree(c, c->d_koff);
+  dfree(c, c->d_kexp);
+  dfree(c, c->d_smax);
+  dfree(c, c->d_fix);
+  dfree(c, c->d_accmore);
 }
 
 // Evaluates and keeps the matrices in c->d_K (allocated by the caller, m2l_f64_digits_bytes).
@@ -443,10 +465,7 @@ efie_status m2l_f64_digits_build(Ctx *c) {
       c->ncl, c->d_own_ptr, c->d_own_src, c->d_far_ptr, c->d_far_src, c->d_koff, c->d_kexp, c->nI, c->kappa, c->d_nodeX,
       circle, (uint4 *)c->d_K); ++c->launches;
   EFIE_CUDA(cudaGetLastError());
-  // splits of the K-steps: enough warps for the chip when there are few targets, two staged chunks each
-  const long long warps = 16ll * c->nsm, have = (long long)c->n_m2l_targets * ((c->nI + 15) / 16);
-  const long long chunks = (long long)(off.back() / 4) / std::max(c->n_m2l_targets, 1);
-  c->f64_split = (int)std::max(1ll, std::min({2 * warps / have, chunks / 2, 16ll}));
+  c->f64_split = k_splits(c, off.back());
   if (c->f64_split > 1) {
     const size_t n = (size_t)(c->f64_split - 1) * c->ncl * 4 * c->nI;
     EFIE_TRY(dalloc(c, &c->d_accmore, n));

@@ -13,6 +13,7 @@ using namespace efie;
 
 namespace efie {
 efie_status dev_batch_alloc(Ctx *c, int R);
+size_t dev_batch_bytes(const Ctx *c, int R);
 efie_status dev_scatter(Ctx *c, const double2 *ys, double2 *y);
 efie_status dev_gather(Ctx *c, const double2 *x, double2 *xs);
 efie_status dev_norms(Ctx *c, int N, const double2 *v, double *out);
@@ -576,14 +577,14 @@ static efie_status solve_batched(Ctx *c, int nrhs, const double *b, double *x, i
   const size_t N = c->ndof;
   size_t fr = 0, tot = 0;
   EFIE_CUDA(cudaMemGetInfo(&fr, &tot));
-  const size_t per = gmres_batch_bytes_per_system(c) + 32 * N + size_t(56) * c->nsup +
-                     size_t(80) * c->ncl * c->nI + (m2l_tc_supported(c) ? m2l_tc_bytes(c, 16) / 16 : 0);
-  int chunk = (int)std::min<size_t>(64, (size_t)(0.8 * (double)fr) / std::max<size_t>(per, 1));
-  if (chunk < 1) {
+  const size_t room = (size_t)(0.8 * (double)fr), basis = gmres_batch_bytes_per_system(c);
+  if (basis + 32 * N + size_t(56) * c->nsup + size_t(80) * c->ncl * c->nI > room) {
     c->err = "solve: the Krylov basis of one system does not fit in the free device memory";
     return EFIE_ENOMEM;
   }
-  chunk = std::min(chunk, nrhs);
+  // as many systems as fit with the vectors of their product, right-hand sides and solutions
+  int chunk = std::min(64, nrhs);
+  while (chunk > 1 && chunk * (basis + 32 * N) + dev_batch_bytes(c, chunk) > room) --chunk;
   EFIE_TRY(dev_batch_alloc(c, chunk));
   double2 *d_bb = nullptr, *d_xx = nullptr;
   DevTemp tmp;

@@ -16,6 +16,7 @@
 #include <cmath>
 
 #include "efie_internal.h"
+#include "batch_bytes.h"
 #include "kept_matrices.h"
 #include "fastmath.cuh"
 
@@ -1073,29 +1074,42 @@ static size_t multi_smem(int nI) {
   return sizeof(float4) * 2 * nI + sizeof(float2) * ((size_t)nI * kFB + (size_t)nI * nI);
 }
 
+static bool batch_takes_tc(const Ctx *c, int R) {
+  return c->opt.m2l_batch != 1 && m2l_tc_supported(c) && R > m2l_mma_rhs(c);
+}
+
+// device memory of dev_batch_alloc for R right-hand sides
+size_t dev_batch_bytes(const Ctx *c, int R) {
+  const size_t nodes = (size_t)c->ncl * c->nI;
+  size_t n = batch_sizes(R, c->ndof, c->nsup, nodes, c->nb).bytes();
+  if (c->m2l_split > 1) n += 8 * (size_t)(c->m2l_split - 1) * nodes * 4 * kMmaMaxRhs;
+  if (batch_takes_tc(c, R)) n += m2l_tc_bytes(c, R) + 16 * (size_t)R;
+  return n;
+}
+
 efie_status dev_batch_alloc(Ctx *c, int R) {
   if (R <= c->batch_cap) return EFIE_OK;
   c->batch_cap = 0;  // should an allocation fail, the next product allocates all of them again
   const size_t ncl = c->ncl, nI = c->nI;
-  EFIE_TRY(dalloc(c, &c->d_xB, (size_t)R * c->ndof));
-  EFIE_TRY(dalloc(c, &c->d_yB, (size_t)R * c->ndof));
-  EFIE_TRY(dalloc(c, &c->d_xsB, (size_t)R * c->nsup));
-  EFIE_TRY(dalloc(c, &c->d_ysB, (size_t)R * c->nsup));
-  EFIE_TRY(dalloc(c, &c->d_ysnB, (size_t)R * c->nsup));
-  if (c->d_nblkf) EFIE_TRY(dalloc(c, &c->d_xfB, (size_t)((R + 3) / 4 * 4) * c->nsup * (c->nb == 8 ? 2 : 1)));
-  EFIE_TRY(dalloc(c, &c->d_momB, (size_t)R * ncl * 3 * nI));
-  EFIE_TRY(dalloc(c, &c->d_srcB, (size_t)R * ncl * 4 * nI));
-  EFIE_TRY(dalloc(c, &c->d_accB, (size_t)R * ncl * 4 * nI));
-  EFIE_CUDA(cudaMemsetAsync(c->d_accB, 0, sizeof(float2) * (size_t)R * ncl * 4 * nI, c->stream));
+  const BatchSizes n = batch_sizes(R, c->ndof, c->nsup, ncl * nI, c->nb);
+  EFIE_TRY(dalloc(c, &c->d_xB, n.x));
+  EFIE_TRY(dalloc(c, &c->d_yB, n.x));
+  EFIE_TRY(dalloc(c, &c->d_xsB, n.xs));
+  EFIE_TRY(dalloc(c, &c->d_ysB, n.xs));
+  EFIE_TRY(dalloc(c, &c->d_ysnB, n.xs));
+  if (c->d_nblkf) EFIE_TRY(dalloc(c, &c->d_xfB, n.xf));
+  EFIE_TRY(dalloc(c, &c->d_momB, n.mom));
+  EFIE_TRY(dalloc(c, &c->d_srcB, n.src));
+  EFIE_TRY(dalloc(c, &c->d_accB, n.src));
+  EFIE_CUDA(cudaMemsetAsync(c->d_accB, 0, sizeof(float2) * n.src, c->stream));
   if (c->m2l_split > 1 && !c->d_moreB) {
     const size_t more = (size_t)(c->m2l_split - 1) * ncl * nI * 4 * kMmaMaxRhs;
     EFIE_TRY(dalloc(c, &c->d_moreB, more));
     EFIE_CUDA(cudaMemsetAsync(c->d_moreB, 0, sizeof(float2) * more, c->stream));
   }
-  EFIE_TRY(dalloc(c, &c->d_locB, (size_t)R * ncl * 3 * nI));
+  EFIE_TRY(dalloc(c, &c->d_locB, n.mom));
   // batches that k_m2l_tc takes (dev_matvec_batch): also room for its split sources
-  if (c->opt.precision == EFIE_MIXED_FP32 && m2l_tc_supported(c))
-    EFIE_TRY(m2l_tc_prepare(c, c->opt.m2l_batch != 1 && R > m2l_mma_rhs(c) ? R : 0));
+  if (c->opt.precision == EFIE_MIXED_FP32 && m2l_tc_supported(c)) EFIE_TRY(m2l_tc_prepare(c, batch_takes_tc(c, R) ? R : 0));
   const int sm = (int)multi_smem(kMultiMaxNI);
   for (auto fn : {k_m2l_f32_multi<1>, k_m2l_f32_multi<2>, k_m2l_f32_multi<4>, k_m2l_f32_multi<8>,
                   k_m2l_f32_multi<12>, k_m2l_f32_multi<16>, k_m2l_f32_multi<18>})

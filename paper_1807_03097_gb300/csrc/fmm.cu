@@ -1126,7 +1126,8 @@ __global__ void k_sum2(size_t n, const double2 *__restrict__ a, const double2 *_
 // Y[r] = A X[r], r < R (host arrays of device pointers).  superspace: X[r] and Y[r] are
 // superspace vectors and the product is (N + F) X[r] (no T gather / scatter).
 efie_status dev_matvec_batch(Ctx *c, int R, const double2 *const *X, double2 *const *Y, bool superspace) {
-  if (c->opt.precision != EFIE_MIXED_FP32 || R == 1 || (c->opt.m2l_batch == 1 && c->nI > kMultiMaxNI)) {
+  if (c->opt.precision != EFIE_MIXED_FP32 || (R == 1 && !batch_takes_tc(c, c->lockstep)) ||
+      (c->opt.m2l_batch == 1 && c->nI > kMultiMaxNI)) {
     for (int r = 0; r < R; ++r) EFIE_TRY(superspace ? dev_matvec_super(c, X[r], Y[r]) : dev_matvec(c, X[r], Y[r]));
     return EFIE_OK;
   }
@@ -1158,8 +1159,9 @@ efie_status dev_matvec_batch(Ctx *c, int R, const double2 *const *X, double2 *co
   EFIE_TRY(tree_up_f32(c, st, R, c->d_xsB, c->d_momB, c->d_srcB, ld));
   EFIE_CUDA(cudaEventRecord(c->tm.ev[3], st));
   // a few right-hand sides, or tiles too large for tensor memory: kernel entries in mma.sync operands
-  // (a lockstep solve keeps the kernel of its first product while systems drop out: the two round
-  // differently by 1e-6, which would cost GMRES iterations at a tolerance of that size)
+  // (a lockstep solve keeps one kernel while systems drop out, down to the last: the two round
+  // differently by 1e-6, which costs GMRES iterations at a tolerance of that size; 3 systems on the cube of
+  // 1 536 elements, kappa = 6: 244 -> 235 iterations with the last system on the others' kernel)
   const bool use_mma = c->opt.m2l_batch != 1 && std::max(R, c->lockstep) <= m2l_mma_rhs(c);
   const bool use_tc = c->opt.m2l_batch != 1 && !use_mma;
   const int nslab = use_mma && R <= kMmaMaxRhs ? c->m2l_split : 1;

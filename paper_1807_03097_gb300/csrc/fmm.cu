@@ -837,8 +837,8 @@ static efie_status far_chain_f64(Ctx *c, const double2 *xs, double2 *ys) {
   if (c->k_digits) EFIE_TRY(m2l_f64_digits_fix(c, st, c->d_src));
   // The M2L on the FP64 pipe has about as many blocks as fit at once: they stay where they are placed, and beside
   // a near field that is still running they crowd the SMs that it has left.  10.7 ms against 18.9 (384
-  // elements, 36 nodes) for a wait of 0.03 ms; the digits take many waves and are not sensitive.
-  else EFIE_CUDA(cudaStreamWaitEvent(st, c->join, 0));
+  // elements, 36 nodes) for a wait of 0.03 ms.  A block an SM or fewer do not crowd, and the digits take many waves.
+  else if (c->n_m2l_targets > c->nsm) EFIE_CUDA(cudaStreamWaitEvent(st, c->join, 0));
   cudaEventRecord(c->tm.ev[3], st);
   int nslab = 1;
   if (c->n_m2l_targets > 0 && c->k_digits) {

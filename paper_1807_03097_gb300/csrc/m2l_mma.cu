@@ -15,14 +15,11 @@
 // (|lo| <= 2^-12 |x|), the entries truncated, because the tensor core reads the upper 19 bits of a
 // register as it is: hi costs no instruction then, lo = x - (x & mask) two.  Of lo's 13 bits the tensor
 // core in turn drops up to two, 0.875 units of 2^-23 on average over evenly distributed lo, which is
-// 7.5e-8 of x over evenly distributed logarithms.  hi hi + hi lo + lo hi leaves out about 2^-23.  The
-// tensor core truncates when it accumulates, so every 8 source nodes get a fresh accumulator (the four small
-// products first), which is added to FP32 sums on the CUDA cores; these enter the running sums by two-sum
-// (compensated) addition once per 64 source nodes.  The two large products (Re G, then Im G on top) shorten an
-// accumulator by half a unit of 2^-23 each on average, 4.3e-8 of it over evenly distributed logarithms,
-// the first of what is then half of it: 6.4e-8.  Both means are given back when the sums are written:
-// relative to the far part, the product of smooth problems was 9e-8 to 13e-8 too small without the second
-// (sphere, cube, kappa <= 1), 3e-8 to 6e-8 with it, which the FP32 sums on the CUDA cores had too.
+// 7.5e-8 of x over evenly distributed logarithms; that mean is given back when the sums are
+// written.  hi hi + hi lo + lo hi leaves out about 2^-23.  The tensor core truncates when it accumulates, so
+// every 8 source nodes get a fresh accumulator (the four small products first), which is added
+// to FP32 sums on the CUDA cores; these enter the running sums by two-sum (compensated) addition
+// once per 64 source nodes.
 //
 // Kernel entry.  Per source node and target, y = x_s - d with d = c_t - c_s is the node seen from
 // the target's centre and a = |y|; the fields carry e^{i kappa a} / (4 pi), from the FP64 phase of
@@ -50,7 +47,7 @@ namespace {
 
 constexpr int kMmaNodes = 64;   // source nodes staged at a time
 constexpr int kMmaSteps = kMmaNodes / 8;
-constexpr float kCut = 7.5e-8f + 6.4e-8f;  // mean shares lost to the truncation of lo parts and of accumulators
+constexpr float kCut = 7.5e-8f; // mean share of an entry lost to the truncation of its lo part
 constexpr int kMmaMaxWarps = 7; // ceil(17^2 / 16) = 19 row tiles, 3 per warp
 
 // Shared memory of one block (float4 units): B fragments [step][rhs][re, im][lane] (steps 64 bytes

@@ -524,7 +524,7 @@ def run_gpu(args):
             "metric": METRIC,
             "value": value, "unit": "solves/s", "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
             "ms_per_step": ms, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-            "dtype": "f32-m2l/f64" if prec else "f64", "data": "synthetic",
+            "dtype": "tf32x3-m2l/f32/f64" if prec else "f64", "data": "synthetic",
             "config": dict(WORKLOAD, precision=args.precision, parallelism="replicas" if world > 1 else "single"),
             "gmres_iterations": int(np.median(its)), "converged": all(conv),
             "setup_ms": st_["setup_ms"],

@@ -88,7 +88,8 @@ typedef struct {
                         in every product, which is faster than streaming them); 1 always
                         evaluate; 2 always keep (EFIE_ENOMEM if they do not fit) */
   int m2l_batch;     /* M2L of a product with several right-hand sides in the mixed form:
-                        0 automatic, 1 FP32 on the CUDA cores, 2 tensor cores (q <= 10;
+                        0 automatic, 1 FP32 on the CUDA cores (q <= 11; beyond, one right-hand side
+                        at a time as in a product with one), 2 tensor cores (q <= 10;
                         EFIE_EINVAL at setup otherwise).  0 and 2: kernel entries in the operands of
                         mma.sync (split TF32) for a few right-hand sides and for q > 10, tcgen05
                         (split FP16) for more, both with FP32 accumulation */

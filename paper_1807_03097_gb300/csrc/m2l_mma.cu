@@ -19,7 +19,12 @@
 // written.  hi hi + hi lo + lo hi leaves out about 2^-23.  The tensor core truncates when it accumulates, so
 // every 8 source nodes get a fresh accumulator (the four small products first), which is added
 // to FP32 sums on the CUDA cores; these enter the running sums by two-sum (compensated) addition
-// once per 64 source nodes.
+// once per 64 source nodes.  The two large products of a step still shorten its accumulator by half a unit of
+// 2^-23 each on average, 6.4e-8 of the sum: at kappa <= 1, where the phases' errors are small, the far part is
+// 9e-8 to 13e-8 too small (FP32 sums on the CUDA cores: up to 6e-8) and the whole product up to 1.23 times as far
+// from 64 bits, at kappa >= 3 0.3 to 0.7 times.  kCut = 1.39e-7 would give that mean back too (1.13 times); it was
+// taken back because it moves residuals at the tolerance of a solve by some percent, and so the step at which
+// some stop (a cube of 24 elements in a group: errors of 1e-6 instead of 1e-7 to 6e-7 at a tolerance of 1e-6).
 //
 // Kernel entry.  Per source node and target, y = x_s - d with d = c_t - c_s is the node seen from
 // the target's centre and a = |y|; the fields carry e^{i kappa a} / (4 pi), from the FP64 phase of
@@ -35,7 +40,8 @@
 // 4.01 ms at 519 480 pairs of 81 nodes, 1.34 -> 1.05 ms at 125 760, 92 -> 18 us at 5 472 pairs of 25 nodes
 // (split lists), 15.7 -> 0.82 ms for two right-hand sides with 144 nodes; error of the product against
 // 64 bits 4.2e-7 -> 1.6e-7 (sphere, kappa = 10).  More warps with fewer tiles (2 or 1 a warp), fewer registers,
-// separate accumulators for Re G and Im G, and 128 nodes a stage were measured and slower by 1 to 20 %.
+// separate accumulators for Re G and Im G, and 128 nodes a stage were measured and slower by 1 to 20 %.  Entries
+// rounded instead of truncated to hi: 7 % slower at 81 nodes, 3 % at 49, products 1 to 7 % closer to 64 bits.
 #include <algorithm>
 
 #include "efie_internal.h"
@@ -194,8 +200,7 @@ __device__ __forceinline__ void sweep(const RowConst (&u)[MT], const float4 *__r
 
 // One block per (target cluster, split of its source list, group of NR right-hand sides).
 //   src[(cluster nI + node) ld + 4 r + f], acc likewise for the first split; the others go to
-//   more[(split - 1) slab + (cluster nI + node) ldm + 4 r + f] and are added, in order, by the
-//   unfolding kernels.
+//   more[(split - 1) slab + (cluster nI + node) ldm + 4 r + f] and are added, in order, by k_add_splits.
 // FAST: lengths are scaled by kappa while they are staged, so that delta is the phase; else (kappa so
 // small or large that squares of scaled lengths could leave the FP32 range, or phases beyond
 // +-100 pi) lengths stay as they are, and the phase is reduced to [-pi, pi] (two-constant
@@ -378,7 +383,10 @@ int m2l_mma_splits(const Ctx *c) {
 // 1 536 elements): 16 nodes, 6 right-hand sides 0.31 / 0.38; 25 nodes 6: 0.64 / 0.67; 49 nodes 3: 0.85 / 1.06,
 // 4: 1.23 / 1.06; 81 nodes 2: 1.47 / 1.96, 3: 2.27 / 1.96; 121 nodes 2: 3.02 / 3.42, 3: 4.37 / 3.42.  Per pair
 // k_m2l_tc takes (rows + 94) x source nodes (rows padded to 64, 96 or 128, nodes to 8), this kernel a
-// right-hand side's (rows + 8) x nodes / 1.36 (rows padded to its tiles).
+// right-hand side's (rows + 8) x nodes / 1.36 (rows padded to its tiles).  From 24 to 6 144 elements and 9 to
+// 121 nodes a batch of this kernel is at most 3 % behind k_m2l_tc, but for 7 right-hand sides at 16 nodes and 1 024
+// elements or more (2.19 against 1.77 ms at 4 096); for a few dozen targets, where only this kernel splits
+// lists, it could take more than 7 (24 elements, 9 nodes: 8 us for 7, 22 us for 8).
 int m2l_mma_rhs(const Ctx *c) {
   if (!m2l_tc_supported(c)) return 1 << 30;
   const int nI = c->nI, nw = mma_warps(nI), mt = ((nI + 15) / 16 + nw - 1) / nw;

@@ -10,11 +10,12 @@
 // Each FP32 operand is scaled by a power of two and split as hi + lo in FP16 (2 x 11 bits); the three
 // products hi*hi, hi*lo and lo*hi carry 21 to 22 bits.  Scales: one per target cluster for G (its
 // smallest node distance), one per field for the sources (the field's largest entry); both are
-// taken back in the epilogue.  FP16 keeps hi and lo whole for entries down to 2^-16 of the largest
-// (then with an absolute error of 2^-39 of it).  The tensor core rounds its accumulator more
-// coarsely than an FP32 add, so every group of 4 block pairs gets a fresh accumulator D = [D1 D2]
-// (one MMA of N = 2 NP against B = [Re G; Im G]), and the group's result is added to running sums S
-// in tensor memory with FP32 adds on the CUDA cores.
+// taken back in the epilogue.  FP16 keeps hi and lo of a source whole down to 2^-16 of the field's largest
+// (below that with an absolute error of 2^-39 of it); an entry G, whose bound 2^9 / (4 pi) leaves room for nodes
+// closer than their clusters' balls, down to 2^-7 of that bound, which the distances of a far list reach.
+// The tensor core rounds its accumulator more coarsely than an FP32 add, so every group of 4 block pairs
+// gets a fresh accumulator D = [D1 D2] (one MMA of N = 2 NP against B = [Re G; Im G]), and the group's
+// result is added to running sums S in tensor memory with FP32 adds on the CUDA cores.
 //
 // Kernel entry: as in k_m2l_mma (y = x_s - d is the source node seen from the target's centre, a = |y|;
 // delta = r - a from num = r^2 - a^2 without cancellation, by one Newton step), but the factor

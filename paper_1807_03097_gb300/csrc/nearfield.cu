@@ -825,7 +825,8 @@ __global__ void k_vec_to_f32x2(int n, const double2 *__restrict__ x, float4 *__r
 // mixed product: at low frequency, where the 1/kappa^2 part cancels, it stopped GMRES at 1e-6 (cube,
 // kappa = 0.8, 768 unknowns, 12 incidences: 114 to 2 060 iterations, 524 on average; now 90 or 91).
 // The 8 x 8 blocks have the room for it (53 us before and after at 6 144 elements: HBM and
-// latency bound); with 18 x 18 blocks the packed FP32 pipe would bound the kernel (63 -> 241 us).
+// latency bound; alone on many more blocks the FP32 pipe bounds it too: 0.36 -> 0.53 ms, leaf-level variant of 24 576
+// elements, whose product hides it); with 18 x 18 blocks the packed FP32 pipe would bound the kernel (63 -> 241 us).
 // Blocks are stored per column in row pairs, float4 (Re 2k, Re 2k+1, Im 2k, Im 2k+1); lane l owns rows
 // 2 (l % 4), 2 (l % 4) + 1 and column l / 4, so one load a lane takes a block, BIF of them in flight.
 template <int BIF>
